@@ -214,10 +214,10 @@ __device__ __forceinline__ T stage_epilogue(const StageArgs<T> &a, long cell, T 
 template <typename T>
 __device__ __forceinline__ void rates2d(const T (&u)[4], T gam, const T (&idx)[3], T &rx, T &ry)
 {
-    T ir = Num<T>::rcp(u[0]);
+    T ir = Num<T>::rcp_ieee(u[0]);
     T vx = u[1] * ir, vy = u[2] * ir;
     T pr = (gam - T(1)) * (u[3] - T(0.5) * (u[1] * vx + u[2] * vy));
-    T c = Num<T>::sqrt(Num<T>::fmax(gam * pr * ir, T(0)));
+    T c = Num<T>::sqrt_ieee(Num<T>::fmax(gam * pr * ir, T(0)));
     rx = (Num<T>::fabs(vx) + c) * idx[0];
     ry = (Num<T>::fabs(vy) + c) * idx[1];
 }
@@ -638,10 +638,10 @@ constexpr size_t stagez_smem_bytes()
 template <typename T>
 __device__ __forceinline__ void rates3d(const T (&u)[5], T gam, const T (&idx)[3], T &rx, T &ry, T &rz)
 {
-    const T ir = Num<T>::rcp(u[0]);
+    const T ir = Num<T>::rcp_ieee(u[0]);
     const T vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
     const T pr = (gam - T(1)) * (u[4] - T(0.5) * (u[1] * vx + u[2] * vy + u[3] * vz));
-    const T c = Num<T>::sqrt(Num<T>::fmax(gam * pr * ir, T(0)));
+    const T c = Num<T>::sqrt_ieee(Num<T>::fmax(gam * pr * ir, T(0)));
     rx = (Num<T>::fabs(vx) + c) * idx[0];
     ry = (Num<T>::fabs(vy) + c) * idx[1];
     rz = (Num<T>::fabs(vz) + c) * idx[2];
@@ -856,10 +856,10 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
                 res[c] = stage_epilogue<T>(a, cell, L, u0, din, lov, dt, (long)NC * nx);
             }
             if (a.rate && a.mode == kModeFinal) {
-                T ir = Num<T>::rcp(res[0]);
+                T ir = Num<T>::rcp_ieee(res[0]);
                 T vx = res[1] * ir;
                 T pr = (tb.gamma - T(1)) * (res[2] - T(0.5) * res[1] * vx);
-                T cc = Num<T>::sqrt(Num<T>::fmax(tb.gamma * pr * ir, T(0)));
+                T cc = Num<T>::sqrt_ieee(Num<T>::fmax(tb.gamma * pr * ir, T(0)));
                 rmx = Num<T>::fmax(rmx, (Num<T>::fabs(vx) + cc) * a.idx[0]);
             }
         }
@@ -877,12 +877,12 @@ __global__ void __launch_bounds__(256) max_rate_kernel(const T *U, long ncell, S
         T u[NC];
 #pragma unroll
         for (int c = 0; c < NC; ++c) u[c] = U[c * ncell + l];
-        T ir = Num<T>::rcp(u[0]);
+        T ir = Num<T>::rcp_ieee(u[0]);
         T m2 = T(0);
 #pragma unroll
         for (int d = 1; d < NC - 1; ++d) m2 = fma(u[d], u[d], m2);
         T pr = (gam - T(1)) * (u[NC - 1] - T(0.5) * m2 * ir);
-        T c = Num<T>::sqrt(Num<T>::fmax(gam * pr * ir, T(0)));
+        T c = Num<T>::sqrt_ieee(Num<T>::fmax(gam * pr * ir, T(0)));
 #pragma unroll
         for (int d = 0; d < NC - 2; ++d) r[d] = Num<T>::fmax(r[d], (Num<T>::fabs(u[1 + d] * ir) + c) * a.idx[d]);
     }
