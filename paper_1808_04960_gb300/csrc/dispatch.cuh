@@ -27,26 +27,32 @@ template <typename T, int R>
 FaceTables<T, R> make_tables(const gpweno_plan_s *p)
 {
     FaceTables<T, R> t;
-    const int S = R + 1;
-    for (int m = 0; m < S; ++m)
-        for (int j = 0; j < S; ++j) {
-            t.wl[m][j] = (T)p->tab.wl[m * S + j];
-            t.wr[m][j] = (T)p->tab.wr[m * S + j];
-            t.gwl[m][j] = (T)p->tab.gwl[m * S + j];
-            t.gwr[m][j] = (T)p->tab.gwr[m * S + j];
-        }
-    for (int k = 0; k < S; ++k)
-        for (int j = 0; j < (R + 2) / 2; ++j) t.Ph[k][j] = (T)p->tab.Ph[k * S + j];
-    for (int m = 0; m < S; ++m) {
-        t.gl[m] = (T)p->tab.gl[m];
-        t.gr[m] = (T)p->tab.gr[m];
-        t.sl1[m] = (T)p->tab.sl1[m];
-        t.sr1[m] = (T)p->tab.sr1[m];
-        t.gsl1[m] = (T)p->tab.gsl1[m];
-        t.gsr1[m] = (T)p->tab.gsr1[m];
-        t.Psum[m] = (T)p->tab.Psum[m];
+    constexpr int S = R + 1, UL = kUnitL<R>, UR = kUnitR<R>;
+    const GpTables &g = p->tab;
+    for (int k = 0; k <= S; ++k) {   // window k: the left side's sub-stencil k, the last one the right side's
+        const double *w = k < S ? g.wl + k * S : g.wr + R * S;
+        for (int j = 0; j < S; ++j) t.w[k][j] = (T)w[j];
+        t.s1[k] = (T)(k < S ? g.sl1[k] : g.sr1[R]);
     }
-    t.eps = (T)p->opts.eps;
+    for (int m = 0; m < S; ++m) {
+        t.gl[m] = (T)(g.gl[m] / g.gl[UL]);
+        t.gr[m] = (T)(g.gr[m] / g.gr[UR - 1]);
+    }
+    const double a1 = g.fa;   // the scale of the smoothness indicators: the first difference's coefficient
+    t.A = (T)(g.fA / a1);
+    t.B = (T)(g.fB / a1);
+    t.D = (T)(g.fD / a1);
+    t.kb = (T)(g.fkb / a1);
+    t.kd = (T)(g.fkd / a1);
+    t.pA = (T)(g.fpA / a1);
+    t.pD = (T)(g.fpD / a1);
+    // eps in that scale; FP32: at least the floor, in the scaled and in the unscaled indicators, so that
+    // (eps + beta)^-2 stays in range
+    const double scale = 1.0 / (a1 * a1);
+    t.eps = (T)std::max(p->opts.eps * scale, (double)Num<T>::kEpsFloor * std::max(scale, 1.0));
+    t.gm1 = (T)(p->gamma - 1.0);
+    t.igm1 = (T)(1.0 / (p->gamma - 1.0));
+    t.hgm1 = (T)(0.5 * (p->gamma - 1.0));
     t.gamma = (T)p->gamma;
     t.p = p->opts.p;
     t.flux = p->opts.flux_form;
@@ -118,6 +124,7 @@ TablesFor<T, R, VAR> make_tables_var(const gpweno_plan_s *p)
             t.Psum3[k] = (T)a.Psum_3[k];
         }
         const double gh = p->opts.ao_gamma_hi, gl = p->opts.ao_gamma_lo;
+        t.eps_ao = (T)p->opts.eps;
         t.g_hi = (T)gh;
         t.g_hi1 = (T)(1.0 - gh);
         t.ig_hi = (T)(1.0 / gh);

@@ -65,7 +65,8 @@ struct Num<float> {
     static __device__ __forceinline__ float pmax(float a, float b) { return fmaxf(a, b); }
     static __device__ __forceinline__ bool positive(float a) { return a > 0.0f; }
     // lower bound of eps + beta in FP32, so that (eps + beta)^-2 stays within range
-    static __device__ __forceinline__ float floored(float eps_beta) { return fmaxf(eps_beta, 1e-18f); }
+    static constexpr float kEpsFloor = 1e-18f;
+    static __device__ __forceinline__ float floored(float eps_beta) { return fmaxf(eps_beta, kEpsFloor); }
     // uncontracted multiply / add (never fused into an FMA, so every kernel rounds alike)
     static __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
     static __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
@@ -118,6 +119,7 @@ struct Num<double> {
     }
     static __device__ __forceinline__ double fmin(double a, double b) { return ::fmin(a, b); }
     // FP64 keeps eps as given (eps > 0)
+    static constexpr double kEpsFloor = 0.0;
     static __device__ __forceinline__ double floored(double eps_beta) { return eps_beta; }
     static __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
     static __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
@@ -126,26 +128,35 @@ struct Num<double> {
 // Weight tables of one plan in the arithmetic type.  Passed by value as a
 // kernel parameter so every (warp-uniform) table read is a constant-bank
 // operand.
+//
+// Window k (k = 0 .. R+1) is cells s-R+k .. s+k of the face's stencil.  The left state's sub-stencil
+// k and the right state's sub-stencil k-1 are the same cells predicted at the same point, so one
+// set of R+2 windows carries both sides' candidates as well as their smoothness indicators.
 template <typename T, int R>
 struct FaceTables {
-    T wl[R + 1][R + 1];   // sub-stencil weights, left state (x* = +1/2 from the stencil of cell s)
-    T wr[R + 1][R + 1];   // sub-stencil weights, right state (x* = -1/2 from the stencil of cell s+1)
-    T gl[R + 1];          // linear weights, left state
-    T gr[R + 1];          // linear weights, right state
-    T sl1[R + 1];         // sum_j wl[m][j] - 1
-    T sr1[R + 1];         // sum_j wr[m][j] - 1
-    T gwl[R + 1][R + 1];  // gl[m] wl[m][j]: the weighted sum of Eq. weight_sum takes one FMA per m
-    T gwr[R + 1][R + 1];  // gr[m] wr[m][j]
-    T gsl1[R + 1];        // gl[m] sl1[m]
-    T gsr1[R + 1];        // gr[m] sr1[m]
-    T Ph[R + 1][(R + 2) / 2];  // P = v / sqrt(lambda) of K_m(sigma), half form, largest lambda first:
-                               // even rows symmetric, odd rows skew (K_m is persymmetric)
-    T Psum[R + 1];        // sum_j of each full row of P (zero for the skew rows)
-    T eps;                // WENO epsilon
+    T w[R + 2][R + 1];    // candidate weights of window k at the face
+    T s1[R + 2];          // sum_j w[k][j] - 1
+    T gl[R + 1];          // linear weights of the left state (windows 0..R) over that of window kUnitL
+    T gr[R + 1];          // linear weights of the right state (windows 1..R+1) over that of window kUnitR
+    // smoothness factor of K_m(sigma), K_m^-1 = sum of squares of five forms of the window's sums
+    // f_j + f_{R-j} and differences f_{R-j} - f_j, divided by the first difference's coefficient
+    // (see window_factors): outer sum (A, B with the inner one or the middle cell), inner (D),
+    // outer difference (1, kb with the inner one), inner (kd)
+    T A, B, D, kb, kd;
+    T pA, pD;             // row sums of the two symmetric forms
+    T eps;                // WENO epsilon in the same scale (FP32: at least the floor of Num<T>)
     T gamma;              // ratio of specific heats
+    T gm1, igm1, hgm1;    // gamma - 1, its inverse and half of it
     int p;                // WENO power, 1 or 2
     int flux;             // face flux: 0 local Lax-Friedrichs, 1 HLLC, 2 HLL
 };
+
+// Window whose linear weight is the unit of each side's weights: the one that is never small
+// against the others for any l/dx >= 1 (ratio at most 3.7), so the scaled sums stay in range.
+template <int R>
+constexpr int kUnitL = R == 2 ? 2 : 1;
+template <int R>
+constexpr int kUnitR = R + 1 - kUnitL<R>;
 
 // Primitive reference state of the "cell-relative" evaluation (normal-first order).
 template <typename T, int NC>
@@ -203,17 +214,21 @@ __device__ __forceinline__ bool prim_pert(const PrimRef<T, NC> &r, const T (&w)[
 //   L_V rows: (0, -an, 0, ap), (1, 0, 0, -ie), e_t, (0, an, 0, ap)
 //   R_V cols: (1, -cr, 0, c^2), (1, 0, 0, 0),   e_t, (1, cr, 0, c^2)
 // with an = rbar/(2c), ap = 1/(2c^2), ie = 1/c^2, cr = c/rbar, rbar = sqrt(rho_L rho_R).
+// With the weight th = sqrt(rho_R) / (sqrt(rho_L) + sqrt(rho_R)) of cell s+1 the Roe velocity is
+// u_s + th du and the Roe enthalpy's sound speed is
+//   c^2 = c_L^2 + th (c_R^2 - c_L^2) + (gamma-1)/2 th (1-th) |du|^2,
+// which needs no enthalpy and only the difference du.
 template <typename T, int NC>
 struct FaceRoe {
     static constexpr int NV = NC - 2, E = NC - 1;
-    T gm1, igm1;
-    T vel[NV];        // Roe velocity
-    T q2;             // |vel|^2
+    T gm1;
+    T th;             // Roe weight of cell s+1
     T c2, c, ic;      // Roe sound speed squared, sound speed, 1/c
     T rbar, irb;      // sqrt(rho_L rho_R) and its inverse
     T an, ie, ap, cr;
     PrimRef<T, NC> ref;
     T Vs[NC];         // primitive state of cell s
+    T dVn[NC];        // V_{s+1} - V_s
     bool ok;          // rho_L, rho_R, c^2 > 0
 
     // row kk of L_V applied to a primitive vector
@@ -225,13 +240,15 @@ struct FaceRoe {
         return v[kk];   // shear: tangential velocity
     }
 
-    // V_j - V_s from the exact conserved difference U_j - U_s by perturbation algebra
-    __device__ __forceinline__ void prim_diff(const T (&uj)[NC], const T (&us)[NC], T (&dV)[NC]) const
+    // Roe velocity
+    __device__ __forceinline__ T vel(int a) const { return fma(th, dVn[1 + a], ref.u[a]); }
+
+    // V_j - V_s from the exact conserved difference U_j - U_s by perturbation algebra (irj = 1/rho_j)
+    __device__ __forceinline__ void prim_diff(const T (&uj)[NC], const T (&us)[NC], T irj, T (&dV)[NC]) const
     {
         T dU[NC];
 #pragma unroll
         for (int a = 0; a < NC; ++a) dU[a] = uj[a] - us[a];
-        const T irj = Num<T>::rcp(uj[0]);
         T k = T(0);
         dV[0] = dU[0];
 #pragma unroll
@@ -242,88 +259,192 @@ struct FaceRoe {
         }
         dV[E] = gm1 * fma(T(-0.5), k, dU[E]);
     }
+    __device__ __forceinline__ void prim_diff(const T (&uj)[NC], const T (&us)[NC], T (&dV)[NC]) const
+    {
+        prim_diff(uj, us, Num<T>::rcp(uj[0]), dV);
+    }
 };
 
-template <typename T, int NC>
-__device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&uR)[NC], T gamma)
+template <typename T, int NC, typename Tables>
+__device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&uR)[NC], const Tables &tb)
 {
     constexpr int NV = NC - 2, E = NC - 1;
     FaceRoe<T, NC> f;
-    f.gm1 = gamma - T(1);
-    f.igm1 = Num<T>::rcp(f.gm1);
+    f.gm1 = tb.gm1;
     const T rL = uL[0], rR = uR[0];
     const T rsL = Num<T>::rsqrt(rL), rsR = Num<T>::rsqrt(rR);
-    const T inv = Num<T>::rcp(rL * rsL + rR * rsR);  // 1/(sqrt(rhoL)+sqrt(rhoR))
-    const T irL = rsL * rsL;
-    T q2 = T(0), mL2 = T(0), mR2 = T(0);
+    const T irL = rsL * rsL, irR = rsR * rsR;
+    f.ref.rho = rL;
+    T mu = T(0);
 #pragma unroll
     for (int a = 0; a < NV; ++a) {
-        f.vel[a] = fma(uL[1 + a], rsL, uR[1 + a] * rsR) * inv;
-        q2 = fma(f.vel[a], f.vel[a], q2);
-        mL2 = fma(uL[1 + a], uL[1 + a], mL2);
-        mR2 = fma(uR[1 + a], uR[1 + a], mR2);
+        f.ref.u[a] = uL[1 + a] * irL;
+        mu = fma(uL[1 + a], f.ref.u[a], mu);
     }
-    const T pL = f.gm1 * fma(T(-0.5) * mL2, irL, uL[E]);
-    const T pR = f.gm1 * fma(T(-0.5) * mR2, rsR * rsR, uR[E]);
-    const T H = fma(uL[E] + pL, rsL, (uR[E] + pR) * rsR) * inv;
-    f.q2 = q2;
-    f.c2 = f.gm1 * fma(T(-0.5), q2, H);
+    f.ref.p = f.gm1 * fma(T(-0.5), mu, uL[E]);
+    f.ref.hp = uL[E] + f.ref.p;
+    f.ref.mn = uL[1];
+    f.Vs[0] = rL;
+#pragma unroll
+    for (int a = 0; a < NV; ++a) f.Vs[1 + a] = f.ref.u[a];
+    f.Vs[E] = f.ref.p;
+    f.prim_diff(uR, uL, irR, f.dVn);
+    const T sL = rL * rsL, sR = rR * rsR;   // sqrt(rho)
+    f.th = sR * Num<T>::rcp(sL + sR);
+    T du2 = T(0);
+#pragma unroll
+    for (int a = 0; a < NV; ++a) du2 = fma(f.dVn[1 + a], f.dVn[1 + a], du2);
+    const T cL2 = tb.gamma * irL * f.ref.p, cR2 = tb.gamma * irR * (f.ref.p + f.dVn[E]);
+    f.c2 = fma(tb.hgm1 * fma(-f.th, f.th, f.th), du2, fma(f.th, cR2 - cL2, cL2));
     f.ok = Num<T>::positive(rL) && Num<T>::positive(rR) && Num<T>::positive(f.c2);
     f.ic = Num<T>::rsqrt(Num<T>::pmax(f.c2, T(1e-30)));
     f.c = f.c2 * f.ic;
-    f.rbar = (rL * rsL) * (rR * rsR);
+    f.rbar = sL * sR;
     f.irb = rsL * rsR;
     f.an = T(0.5) * f.rbar * f.ic;
     f.ie = f.ic * f.ic;
     f.ap = T(0.5) * f.ie;
     f.cr = f.c * f.irb;
-    f.ref.rho = rL;
-#pragma unroll
-    for (int a = 0; a < NV; ++a) f.ref.u[a] = uL[1 + a] * irL;
-    f.ref.p = pL;
-    f.ref.hp = uL[E] + pL;
-    f.ref.mn = uL[1];
-    f.Vs[0] = rL;
-#pragma unroll
-    for (int a = 0; a < NV; ++a) f.Vs[1 + a] = f.ref.u[a];
-    f.Vs[E] = pL;
     return f;
 }
 
-// (eps + beta)^-p of one smoothness window: beta = sum_h (P_h . (f - shift))^2
-// (Eq. beta-eigen) over the window f[w..w+R] of data f_j = f_c + d_j with
-// d_R = 0 (relative to the face's cell s).  pf_h = (f_c - shift) sum_j P_hj is
-// supplied by the caller (zero for the skew rows, whose sums vanish); rows are
-// evaluated in the symmetric/skew half form.
-template <typename T, int R, int NS>
-__device__ __forceinline__ T beta_weight(const FaceTables<T, R> &tb, const T (&d)[NS], int w, const T (&pf)[R + 1])
+// Arithmetic of one characteristic field (T) or of two at once (float2: packed fma/add/mul .f32x2
+// of sm_100 and later, each lane rounded as the scalar operation).
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) { return __ffma2_rn(f2(a), b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float a, float2 b) { return __fmul2_rn(f2(a), b); }
+__device__ __forceinline__ float vrcp(float a) { return Num<float>::rcp(a); }
+__device__ __forceinline__ double vrcp(double a) { return Num<double>::rcp(a); }
+__device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(Num<float>::rcp(a.x), Num<float>::rcp(a.y)); }
+template <typename V>
+__device__ __forceinline__ V vset(double x) { return V(x); }
+template <>
+__device__ __forceinline__ float2 vset<float2>(double x) { return f2((float)x); }
+__device__ __forceinline__ float vcast(float x, float) { return x; }
+__device__ __forceinline__ double vcast(double x, double) { return x; }
+__device__ __forceinline__ float2 vcast(float x, float2) { return f2(x); }
+
+// (eps + beta)^-p of one smoothness window: beta = f^T K_m(sigma)^-1 f (Eq. beta-eigen, in another
+// orthogonal basis) over the window f[w..w+R] of data f_j - shift = d_j + (f_c - shift), with
+// d_R = 0 (relative to the face's cell s).  pA, pD = (f_c - shift) times the row sums of the two
+// symmetric forms, supplied by the caller (the differences' row sums vanish).  Triangular forms
+// (window_factors) and the unit coefficient of the first difference save 2 (R = 2) and 3 (R = 3)
+// of 10 and 16 instructions per window against the eigenvector rows.
+template <typename T, int R, typename V, int NS>
+__device__ __forceinline__ V beta_weight(const FaceTables<T, R> &tb, const V (&d)[NS], int w, V pA, V pD)
 {
-    constexpr int S = R + 1, HALF = S / 2;
-    T ps[HALF > 0 ? HALF : 1], ms[HALF > 0 ? HALF : 1];
-#pragma unroll
-    for (int j = 0; j < HALF; ++j) {
-        const int lo = w + j, hi = w + S - 1 - j;
-        ps[j] = lo == R ? d[hi] : (hi == R ? d[lo] : d[lo] + d[hi]);
-        ms[j] = lo == R ? -d[hi] : (hi == R ? d[lo] : d[lo] - d[hi]);
-    }
-    T beta = tb.eps;   // (eps + beta), accumulated from eps
-#pragma unroll
-    for (int h = 0; h < S; ++h) {
-        T dot;
-        if (h % 2 == 0) {
-            dot = pf[h];
-            if (S % 2 == 1 && w + HALF != R) dot = fma(tb.Ph[h][HALF], d[w + HALF], dot);
-#pragma unroll
-            for (int j = 0; j < HALF; ++j) dot = fma(tb.Ph[h][j], ps[j], dot);
-        } else {
-            dot = tb.Ph[h][0] * ms[0];
-#pragma unroll
-            for (int j = 1; j < HALF; ++j) dot = fma(tb.Ph[h][j], ms[j], dot);
+    // sum and difference of the window's cells j and R-j; `flip` picks the sign of all differences of a
+    // window (their squares are used) so that a term with d_R = 0 is a plain copy
+    const bool flip = w + R == R || (R == 3 && w + 2 == R);
+    auto sum = [&](int j) {
+        const int lo = w + j, hi = w + R - j;
+        return lo == R ? d[hi] : (hi == R ? d[lo] : vadd(d[lo], d[hi]));
+    };
+    auto diff = [&](int j) {
+        const int lo = flip ? w + R - j : w + j, hi = flip ? w + j : w + R - j;
+        return lo == R ? d[hi] : vsub(d[hi], d[lo]);
+    };
+    V beta = vcast(tb.eps, V());   // (eps + beta), accumulated from eps
+    V s = vfma(tb.A, sum(0), pA), k = diff(0);
+    if constexpr (R == 2) {
+        V m = pD;
+        if (w + 1 != R) {
+            s = vfma(tb.B, d[w + 1], s);
+            m = vfma(tb.D, d[w + 1], m);
         }
-        beta = fma(dot, dot, beta);
+        beta = vfma(m, m, beta);
     }
-    const T x = Num<T>::rcp(Num<T>::floored(beta));
-    return tb.p == 2 ? Num<T>::mul_rn(x, x) : x;
+    if constexpr (R == 3) {
+        const V si = sum(1), ki = diff(1);
+        s = vfma(tb.B, si, s);
+        const V m = vfma(tb.D, si, pD), n = vmul(tb.kd, ki);
+        k = vfma(tb.kb, ki, k);
+        beta = vfma(m, m, beta);
+        beta = vfma(n, n, beta);
+    }
+    beta = vfma(k, k, beta);
+    beta = vfma(s, s, beta);
+    const V x = vrcp(beta);
+    return tb.p == 2 ? vmul(x, x) : x;
+}
+
+// Left and right GP-WENO states of a face in one characteristic field (or two, V = float2) from the
+// data d_j relative to cell s (d_R = 0) and the value fc of cell s:
+//   qL = q_L - f_s,  qR = q_R - f_{s+1}.
+// Window k's candidate relative to cell s is q_k = sum_j w_kj d_{k+j} + fc (sum_j w_kj - 1), shared by
+// both sides, and omega_m ~ gamma_m x_k with x_k = (eps + beta_k)^-p (Eq. weights); sum_m omega_m = 1
+// is used exactly.  With the zero mean x_k and x_k q_k are shared too.  MEAN: the left side's windows
+// shift by its centre, cell s (no shift), the right side's by cell s+1 (shift d_{R+1}).
+template <typename T, int R, bool MEAN, typename V, int NS>
+__device__ __forceinline__ void weno_states(const FaceTables<T, R> &tb, const V (&d)[NS], V fc, V &qL, V &qR)
+{
+    constexpr int UL = kUnitL<R>, UR = kUnitR<R>;
+    const V zero = vset<V>(0.0);
+    const V lA = MEAN ? zero : vmul(tb.pA, fc), lD = MEAN ? zero : vmul(tb.pD, fc);
+    const V rA = MEAN ? vmul(-tb.pA, d[R + 1]) : lA, rD = MEAN ? vmul(-tb.pD, d[R + 1]) : lD;
+    V numL, denL, numR, denR;
+    // the windows with a unit weight first, so that each side's sums start without a multiply
+    auto window = [&](int k, V &xl, V &xr, V &tl, V &tr) {
+        V q = vmul(tb.s1[k], fc);
+#pragma unroll
+        for (int j = 0; j <= R; ++j)
+            if (k + j != R) q = vfma(tb.w[k][j], d[k + j], q);
+        if (k <= R) {
+            xl = beta_weight<T, R>(tb, d, k, lA, lD);
+            tl = vmul(xl, q);
+        }
+        if (k > 0) {
+            if (MEAN || k > R) {
+                xr = beta_weight<T, R>(tb, d, k, rA, rD);
+                tr = vmul(xr, q);
+            } else {
+                xr = xl;
+                tr = tl;
+            }
+        }
+    };
+    V xl, xr, tl, tr;
+    window(UL, xl, xr, tl, tr);
+    numL = tl;
+    denL = xl;
+    if constexpr (UR == UL) {
+        numR = tr;
+        denR = xr;
+    } else {
+        V yl, yr, ul, ur;
+        window(UR, yl, yr, ul, ur);
+        numL = vfma(tb.gl[UR], ul, numL);
+        denL = vfma(tb.gl[UR], yl, denL);
+        numR = vfma(tb.gr[UL - 1], tr, ur);
+        denR = vfma(tb.gr[UL - 1], xr, yr);
+    }
+#pragma unroll
+    for (int k = 0; k <= R + 1; ++k) {
+        if (k == UL || k == UR) continue;
+        window(k, xl, xr, tl, tr);
+        if (k <= R) {
+            numL = vfma(tb.gl[k], tl, numL);
+            denL = vfma(tb.gl[k], xl, denL);
+        }
+        if (k > 0) {
+            numR = vfma(tb.gr[k - 1], tr, numR);
+            denR = vfma(tb.gr[k - 1], xr, denR);
+        }
+    }
+    qL = vmul(numL, vrcp(denL));
+    qR = vsub(vmul(numR, vrcp(denR)), d[R + 1]);
 }
 
 // GP-AO tables (Appendix A) on top of the GP-WENO ones: R = 2 serves AO(2,3),
@@ -341,6 +462,7 @@ struct AoFaceTables : FaceTables<T, R> {
     T Phi[NH][(NH + 1) / 2], Psum_hi[NH];
     T Plo[NL][(NL + 1) / 2], Psum_lo[NL];
     T P3[3][2], Psum3[3];
+    T eps_ao;               // WENO epsilon (unscaled)
     T g_hi, g_hi1, ig_hi;   // gamma_HI, 1 - gamma_HI, 1 / gamma_HI
     T g3[3];                // gamma_m = ((1-gHI)(1-gLO)/2, (1-gHI) gLO, (1-gHI)(1-gLO)/2)
 };
@@ -435,7 +557,7 @@ __device__ __forceinline__ T ao_side(const AoFaceTables<T, R> &ta, const T (&d)[
             for (int j = 0; j < 3; ++j)
                 if (w0 + j != R) q = fma(RIGHT ? ta.w3r[m][j] : ta.w3l[m][j], d[w0 + j], q);
             q3[m] = q;
-            x3[m] = inv_pow<T>(ta.eps, T(0.5) * beta_window<T, 3, R, NS>(ta.P3, d, w0, pf), ta.p);
+            x3[m] = inv_pow<T>(ta.eps_ao, T(0.5) * beta_window<T, 3, R, NS>(ta.P3, d, w0, pf), ta.p);
         }
     }
     T pfh[NH];
@@ -445,7 +567,7 @@ __device__ __forceinline__ T ao_side(const AoFaceTables<T, R> &ta, const T (&d)[
 #pragma unroll
     for (int j = 0; j < NH; ++j)
         if (o + j != R) qh = fma(RIGHT ? ta.whr[j] : ta.whl[j], d[o + j], qh);
-    const T xh = inv_pow<T>(ta.eps, T(0.5) * beta_window<T, NH, R, NS>(ta.Phi, d, o, pfh), ta.p);
+    const T xh = inv_pow<T>(ta.eps_ao, T(0.5) * beta_window<T, NH, R, NS>(ta.Phi, d, o, pfh), ta.p);
     const T q_hi = ao_hybrid<T, R>(ta, qh, xh, q3, x3);
     if constexpr (R == 2) {
         return q_hi;
@@ -457,7 +579,7 @@ __device__ __forceinline__ T ao_side(const AoFaceTables<T, R> &ta, const T (&d)[
 #pragma unroll
         for (int j = 0; j < NL; ++j)
             if (o + 1 + j != R) ql = fma(RIGHT ? ta.wlr[j] : ta.wll[j], d[o + 1 + j], ql);
-        const T xl = inv_pow<T>(ta.eps, T(0.5) * beta_window<T, NL, R, NS>(ta.Plo, d, o + 1, pfl), ta.p);
+        const T xl = inv_pow<T>(ta.eps_ao, T(0.5) * beta_window<T, NL, R, NS>(ta.Plo, d, o + 1, pfl), ta.p);
         const T q_lo = ao_hybrid<T, R>(ta, ql, xl, q3, x3);
         const T vh = ta.g_hi * xh, vl = ta.g_hi1 * xl;
         const T inv = Num<T>::rcp(vh + vl);
@@ -466,55 +588,14 @@ __device__ __forceinline__ T ao_side(const AoFaceTables<T, R> &ta, const T (&d)[
     }
 }
 
-// Packed FP32: two characteristic fields per instruction (fma/add/mul .f32x2
-// of sm_100 and later).  Each lane rounds exactly as the scalar operation.
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }
-
-// beta_weight for two fields at once: (eps + beta)^-p of window d[w..w+R] in each lane.
-template <int R, int NS>
-__device__ __forceinline__ float2 beta_weight2(const FaceTables<float, R> &tb, const float2 (&d)[NS], int w,
-                                               const float2 (&pf)[R + 1])
-{
-    constexpr int S = R + 1, HALF = S / 2;
-    float2 ps[HALF > 0 ? HALF : 1], ms[HALF > 0 ? HALF : 1];
-#pragma unroll
-    for (int j = 0; j < HALF; ++j) {
-        const int lo = w + j, hi = w + S - 1 - j;
-        ps[j] = lo == R ? d[hi] : (hi == R ? d[lo] : add2(d[lo], d[hi]));
-        ms[j] = lo == R ? mul2(d[hi], f2(-1.0f)) : (hi == R ? d[lo] : sub2(d[lo], d[hi]));
-    }
-    float2 beta = f2(tb.eps);   // (eps + beta), accumulated from eps
-#pragma unroll
-    for (int h = 0; h < S; ++h) {
-        float2 dot;
-        if (h % 2 == 0) {
-            dot = pf[h];
-            if (S % 2 == 1 && w + HALF != R) dot = fma2(f2(tb.Ph[h][HALF]), d[w + HALF], dot);
-#pragma unroll
-            for (int j = 0; j < HALF; ++j) dot = fma2(f2(tb.Ph[h][j]), ps[j], dot);
-        } else {
-            dot = mul2(f2(tb.Ph[h][0]), ms[0]);
-#pragma unroll
-            for (int j = 1; j < HALF; ++j) dot = fma2(f2(tb.Ph[h][j]), ms[j], dot);
-        }
-        beta = fma2(dot, dot, beta);
-    }
-    const float2 x = make_float2(Num<float>::rcp(Num<float>::floored(beta.x)),
-                                 Num<float>::rcp(Num<float>::floored(beta.y)));
-    return tb.p == 2 ? mul2(x, x) : x;
-}
-
 // One face, cell-relative form.  st[0..2R+1] is the normal-first conserved
 // stencil; the face s+1/2 lies between st[R] (cell s) and st[R+1] (cell s+1).
 // Outputs
-//   A = F_{s+1/2} - F(U_s)      (numerical face flux relative to cell s)
-//   B = F(U_{s+1}) - F(U_s)     (physical flux difference of the two cells)
-// so that the flux jump across cell s, F_{s+1/2} - F_{s-1/2} = A_s - A_{s-1} + B_{s-1},
-// is formed from small quantities only.  In real arithmetic this is exactly
+//   A = 2 (F_{s+1/2} - F(U_s))      (numerical face flux relative to cell s)
+//   M = 2 (F_{s+1/2} - F(U_{s+1}))  (relative to cell s+1)
+// so that the flux jump across cell s, F_{s+1/2} - F_{s-1/2} = (A_s - M_{s-1}) / 2,
+// is formed from small quantities only (the factor 2 spares the halving of the
+// Lax-Friedrichs mean; the divergence's weights take it back).  In real arithmetic this is exactly
 // the scheme: characteristic variables of the primitive variables
 // V = (rho, u, p) with the eigenvectors of the primitive system at the Roe
 // average of cells s, s+1 (Section 6; "FD-Primitive"), GP-WENO states by
@@ -528,26 +609,30 @@ __device__ __forceinline__ float2 beta_weight2(const FaceTables<float, R> &tb, c
 //     V_{s+1} + R (q_R - L V_{s+1}), using R L = I and sum_m omega_m = 1;
 //   * fluxes and conserved states are perturbations about V_s (prim_pert).
 // Returns false on a non-physical Roe, left, right or neighbour state.
+// Bound: instruction issue and the FP32 pipe (FP32), the FP64 pipe (FP64), so the count of
+// arithmetic instructions.  Sharing the candidates of a window between both sides, triangular
+// smoothness forms, the Roe sound speed and the neighbour flux from differences, and doubled fluxes
+// measured per step against the form without them: FP32 1024^2 R = 2 232 -> 205 us, 4096^2
+// 2848 -> 2460 us, 3D 512^3 R = 3 63.1 -> 53.4 ms; FP64 512^2 R = 2 3086 -> 2702 us.
 template <typename T, int NC, int R, bool MEAN = false, bool AO = false>
 __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                         T (&B)[NC])
+                                         T (&M)[NC])
 {
     constexpr int NS = 2 * R + 2;
     constexpr int E = NC - 1;
-    constexpr int S = R + 1;
-    const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb.gamma);
+    const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
     bool ok = f.ok;
-    const T igm1 = f.igm1, c = f.c, c2 = f.c2, cr = f.cr;
+    const T igm1 = tb.igm1, c = f.c, c2 = f.c2, cr = f.cr;
     const PrimRef<T, NC> &ref = f.ref;
-    const T(&vel)[NC - 2] = f.vel;
+    const T(&dn)[NC] = f.dVn;
 
     // primitive differences V_j - V_s from the exact conserved differences
     T dV[NS][NC];
 #pragma unroll
     for (int j = 0; j < NS; ++j) {
-        if (j == R) {
+        if (j == R || j == R + 1) {
 #pragma unroll
-            for (int a = 0; a < NC; ++a) dV[j][a] = T(0);
+            for (int a = 0; a < NC; ++a) dV[j][a] = j == R ? T(0) : dn[a];
             continue;
         }
         f.prim_diff(st[j], st[R], dV[j]);
@@ -565,43 +650,17 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
         for (int k0 = 0; k0 + 1 < NC; k0 += 2) {
             const int k1 = k0 + 1;
             const float2 fc = make_float2(f.lrow(k0, f.Vs), f.lrow(k1, f.Vs));
-            float2 d[NS];
+            float2 d[NS], qL, qR;
 #pragma unroll
             for (int j = 0; j < NS; ++j)
                 d[j] = (j == R) ? f2(0.0f) : make_float2(f.lrow(k0, dV[j]), f.lrow(k1, dV[j]));
-            float2 pfl[S], pfr[S];
-#pragma unroll
-            for (int h = 0; h < S; ++h) {
-                pfl[h] = (h % 2 == 0 && !MEAN) ? mul2(f2(tb.Psum[h]), fc) : f2(0.0f);
-                pfr[h] = (h % 2 == 0) ? (MEAN ? mul2(f2(-tb.Psum[h]), d[R + 1]) : pfl[h]) : f2(0.0f);
-            }
-            float2 numL = f2(0.0f), denL = f2(0.0f), numR = f2(0.0f), denR = f2(0.0f);
-            float2 xl = beta_weight2<R, NS>(tb, d, 0, pfl);
-#pragma unroll
-            for (int m = 0; m <= R; ++m) {
-                const float2 xr = beta_weight2<R, NS>(tb, d, m + 1, pfr);
-                // gamma_m (candidate_m - centre), with gamma folded into the tables
-                float2 sl = mul2(f2(tb.gsl1[m]), fc), sr = mul2(f2(tb.gsr1[m]), fc);
-#pragma unroll
-                for (int j = 0; j <= R; ++j) {
-                    if (m + j != R) sl = fma2(f2(tb.gwl[m][j]), d[m + j], sl);
-                    if (1 + m + j != R) sr = fma2(f2(tb.gwr[m][j]), d[1 + m + j], sr);
-                }
-                numL = fma2(xl, sl, numL);
-                denL = fma2(f2(tb.gl[m]), xl, denL);
-                numR = fma2(xr, sr, numR);
-                denR = fma2(f2(tb.gr[m]), xr, denR);
-                if (m < R) xl = MEAN ? beta_weight2<R, NS>(tb, d, m + 1, pfl) : xr;
-            }
-            const float2 qL = mul2(numL, make_float2(Num<float>::rcp(denL.x), Num<float>::rcp(denL.y)));
-            const float2 qR = sub2(mul2(numR, make_float2(Num<float>::rcp(denR.x), Num<float>::rcp(denR.y))), d[R + 1]);
+            weno_states<T, R, MEAN>(tb, d, fc, qL, qR);
             dqL[k0] = qL.x;
             dqR[k0] = qR.x;
             dqL[k1] = qL.y;
             dqR[k1] = qR.y;
         }
     }
-    {
 #pragma unroll
     for (int kk = kScalarFrom; kk < NC; ++kk) {
         const T fc = f.lrow(kk, f.Vs);
@@ -614,71 +673,48 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
             dqL[kk] = ao_side<T, R, NS, false, MEAN>(ta, d, fc);                 // q_L - L V_s
             dqR[kk] = ao_side<T, R, NS, true, MEAN>(ta, d, fc) - d[R + 1];      // q_R - L V_{s+1}
         } else {
-            // zero mean: both sides shift by f_c, so the right side's window m is the
-            // left side's window m+1 and the R+2 windows are shared.  Mean f_centre:
-            // the left side's centre is cell s (no shift), the right side's is cell
-            // s+1 (shift by d_{R+1}), and the 2R+2 windows are separate.
-            T pfl[S], pfr[S];
-#pragma unroll
-            for (int h = 0; h < S; ++h) {
-                pfl[h] = (h % 2 == 0 && !MEAN) ? tb.Psum[h] * fc : T(0);
-                pfr[h] = (h % 2 == 0) ? (MEAN ? -tb.Psum[h] * d[R + 1] : pfl[h]) : T(0);
-            }
-            // --- candidates relative to the centre cells and nonlinear weights ---
-            // omega_m ~ gamma_m (eps + beta_m)^-p  (Eq. weights); sum_m omega_m = 1 is used exactly.
-            T numL = T(0), denL = T(0), numR = T(0), denR = T(0);
-            T xl = beta_weight<T, R, NS>(tb, d, 0, pfl);
-#pragma unroll
-            for (int m = 0; m <= R; ++m) {
-                const T xr = beta_weight<T, R, NS>(tb, d, m + 1, pfr);
-                T sl = tb.gsl1[m] * fc, sr = tb.gsr1[m] * fc;   // gamma_m (candidate_m - centre)
-#pragma unroll
-                for (int j = 0; j <= R; ++j) {
-                    if (m + j != R) sl = fma(tb.gwl[m][j], d[m + j], sl);
-                    if (1 + m + j != R) sr = fma(tb.gwr[m][j], d[1 + m + j], sr);
-                }
-                numL = fma(xl, sl, numL);
-                denL = fma(tb.gl[m], xl, denL);
-                numR = fma(xr, sr, numR);
-                denR = fma(tb.gr[m], xr, denR);
-                if (m < R) xl = MEAN ? beta_weight<T, R, NS>(tb, d, m + 1, pfl) : xr;
-            }
-            dqL[kk] = numL * Num<T>::rcp(denL);              // q_L - L V_s
-            dqR[kk] = numR * Num<T>::rcp(denR) - d[R + 1];   // q_R - L V_{s+1}
+            weno_states<T, R, MEAN>(tb, d, fc, dqL[kk], dqR[kk]);
         }
-    }
     }
 
     // --- back-projection: primitive states relative to cell s -------------
     T wL[NC], wR[NC];
     wL[0] = dqL[0] + dqL[1] + dqL[E];
-    wR[0] = dV[R + 1][0] + (dqR[0] + dqR[1] + dqR[E]);
+    wR[0] = dn[0] + (dqR[0] + dqR[1] + dqR[E]);
     wL[1] = cr * (dqL[E] - dqL[0]);
-    wR[1] = fma(cr, dqR[E] - dqR[0], dV[R + 1][1]);
+    wR[1] = fma(cr, dqR[E] - dqR[0], dn[1]);
 #pragma unroll
     for (int a = 2; a < E; ++a) {
         wL[a] = dqL[a];
-        wR[a] = dV[R + 1][a] + dqR[a];
+        wR[a] = dn[a] + dqR[a];
     }
     wL[E] = c2 * (dqL[0] + dqL[E]);
-    wR[E] = fma(c2, dqR[0] + dqR[E], dV[R + 1][E]);
+    wR[E] = fma(c2, dqR[0] + dqR[E], dn[E]);
 
     // --- face flux relative to F(U_s), and F(U_{s+1}) - F(U_s) ---------------
-    T GL[NC], GR[NC], cL[NC], cR[NC], cB[NC], uL, uR, aL, aR, uB, aB;
+    T GL[NC], GR[NC], cL[NC], cR[NC], B[NC], uL, uR, aL, aR;
     ok = prim_pert<T, NC>(ref, wL, tb.gamma, igm1, GL, cL, uL, aL) && ok;
     ok = prim_pert<T, NC>(ref, wR, tb.gamma, igm1, GR, cR, uR, aR) && ok;
-    T dn[NC];
+    // B = F(U_{s+1}) - F(U_s) from the exact conserved difference and the primitive one:
+    // (dm_n, u'_n dm_n + m_n du_n + dp, u'_t dm_n + m_n du_t, hp du_n + u'_n (dE + dp)), u' = u_{s+1}
+    {
+        const T dm = st[R + 1][1] - st[R][1], un = ref.u[0] + dn[1];
+        B[0] = dm;
+        B[1] = fma(dm, un, fma(ref.mn, dn[1], dn[E]));
 #pragma unroll
-    for (int a = 0; a < NC; ++a) dn[a] = dV[R + 1][a];
-    ok = prim_pert<T, NC>(ref, dn, tb.gamma, igm1, B, cB, uB, aB) && ok;
+        for (int a = 2; a < E; ++a) B[a] = fma(dm, ref.u[a - 1] + dn[a], ref.mn * dn[a]);
+        B[E] = fma(dn[1], ref.hp, un * ((st[R + 1][E] - st[R][E]) + dn[E]));
+        ok = ok && Num<T>::positive(ref.p + dn[E]);
+    }
     if (tb.flux == 1) {
         // HLLC with Einfeldt speeds from the Roe average.  The contact speed enters only
         // through S* - u_K = (dp - rho_K' (S_K' - u_K') du) / D (K' the other side), formed
         // from the small differences dp = p_R - p_L, du = u_R - u_L, so the star states
         // U*_K - U_K stay accurate increments.
+        const T vel0 = f.vel(0);
         const T rhoL = ref.rho + wL[0], rhoR = ref.rho + wR[0];
         const T pLf = ref.p + wL[E], pRf = ref.p + wR[E];
-        const T SL = Num<T>::fmin(uL - aL, vel[0] - c), SR = Num<T>::fmax(uR + aR, vel[0] + c);
+        const T SL = Num<T>::fmin(uL - aL, vel0 - c), SR = Num<T>::fmax(uR + aR, vel0 + c);
         const T mL = rhoL * (SL - uL), mR = rhoR * (SR - uR);
         const T iD = Num<T>::rcp(mL - mR);
         const T dp = wR[E] - wL[E], du = wR[1] - wL[1];
@@ -708,13 +744,14 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
             else if (SR <= T(0)) f = GR[a];
             else if (Ss >= T(0)) f = fma(SL, dUL[a], GL[a]);
             else f = fma(SR, dUR[a], GR[a]);
-            A[a] = f;
+            A[a] = T(2) * f;
         }
     } else if (tb.flux == 2) {
         // HLL with the same Einfeldt speeds: F_L if S_L >= 0, F_R if S_R <= 0, else
         // (S_R F_L - S_L F_R + S_L S_R (U_R - U_L)) / (S_R - S_L); relative to F(U_s)
         // the flux terms keep that form with G_K = F_K - F(U_s) and c_K = U_K - U_s.
-        const T SL = Num<T>::fmin(uL - aL, vel[0] - c), SR = Num<T>::fmax(uR + aR, vel[0] + c);
+        const T vel0 = f.vel(0);
+        const T SL = Num<T>::fmin(uL - aL, vel0 - c), SR = Num<T>::fmax(uR + aR, vel0 + c);
         const T iS = Num<T>::rcp(SR - SL);
 #pragma unroll
         for (int a = 0; a < NC; ++a) {
@@ -722,18 +759,54 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
             if (SL >= T(0)) f = GL[a];
             else if (SR <= T(0)) f = GR[a];
             else f = (fma(SR, GL[a], -SL * GR[a]) + SL * SR * (cR[a] - cL[a])) * iS;
-            A[a] = f;
+            A[a] = T(2) * f;
         }
     } else {
         const T alpha = Num<T>::pmax(Num<T>::fabs(uL) + aL, Num<T>::fabs(uR) + aR);
 #pragma unroll
-        for (int a = 0; a < NC; ++a) A[a] = T(0.5) * ((GL[a] + GR[a]) - alpha * (cR[a] - cL[a]));
+        for (int a = 0; a < NC; ++a) A[a] = fma(-alpha, cR[a] - cL[a], GL[a] + GR[a]);
     }
+#pragma unroll
+    for (int a = 0; a < NC; ++a) M[a] = fma(T(-2), B[a], A[a]);
     return ok;
 }
 
-// One face of the FD-Flux form (Section 2), cell-relative; outputs as face_rel:
-//   A = f^_{s+1/2} - F(U_s),  B = F(U_{s+1}) - F(U_s).
+// Sum of the two reconstructed parts of one field (or two) of the FD-Flux form, relative to cell s:
+// the left part from p (relative to its cell-s value fcp) on windows 0..R, the right part from m
+// (fcm) on windows 1..R+1.  Zero mean: shifts fcp and fcm; MEAN: centres cell s and cell s+1.
+template <typename T, int R, bool MEAN, typename V, int NS>
+__device__ __forceinline__ V fdf_state(const FaceTables<T, R> &tb, const V (&p)[NS], const V (&m)[NS], V fcp, V fcm)
+{
+    constexpr int UL = kUnitL<R>, UR = kUnitR<R>;
+    const V zero = vset<V>(0.0);
+    const V lA = MEAN ? zero : vmul(tb.pA, fcp), lD = MEAN ? zero : vmul(tb.pD, fcp);
+    const V rA = MEAN ? vmul(-tb.pA, m[R + 1]) : vmul(tb.pA, fcm), rD = MEAN ? vmul(-tb.pD, m[R + 1]) : vmul(tb.pD, fcm);
+    auto part = [&](const V(&d)[NS], V fc, int k, V sA, V sD, V &x) {
+        V q = vmul(tb.s1[k], fc);
+#pragma unroll
+        for (int j = 0; j <= R; ++j)
+            if (k + j != R) q = vfma(tb.w[k][j], d[k + j], q);
+        x = beta_weight<T, R>(tb, d, k, sA, sD);
+        return vmul(x, q);
+    };
+    V denL, denR, x;
+    V numL = part(p, fcp, UL, lA, lD, denL), numR = part(m, fcm, UR, rA, rD, denR);
+#pragma unroll
+    for (int k = 0; k <= R + 1; ++k) {
+        if (k <= R && k != UL) {
+            numL = vfma(tb.gl[k], part(p, fcp, k, lA, lD, x), numL);
+            denL = vfma(tb.gl[k], x, denL);
+        }
+        if (k > 0 && k != UR) {
+            numR = vfma(tb.gr[k - 1], part(m, fcm, k, rA, rD, x), numR);
+            denR = vfma(tb.gr[k - 1], x, denR);
+        }
+    }
+    return vfma(numL, vrcp(denL), vmul(numR, vrcp(denR)));
+}
+
+// One face of the FD-Flux form (Section 2), cell-relative; outputs as face_rel without the factor 2:
+//   A = f^_{s+1/2} - F(U_s),  M = f^_{s+1/2} - F(U_{s+1}).
 // The point fluxes are cell averages of the function whose face values are
 // the numerical fluxes (Eqs. prim_F, design).  They are split by local
 // Lax-Friedrichs, F+- = (F +- alpha U)/2 with alpha the largest |u_n| + c over
@@ -750,10 +823,16 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
 // projects back to F(U_s).  Returns false on a non-physical state.
 template <typename T, int NC, int R, bool MEAN = false>
 __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                         T (&B)[NC])
+                                         T (&M)[NC])
 {
-    constexpr int NS = 2 * R + 2, E = NC - 1, NV = NC - 2, S = R + 1;
-    const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb.gamma);
+    constexpr int NS = 2 * R + 2, E = NC - 1, NV = NC - 2;
+    const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
+    T vel[NV], q2 = T(0), B[NC];
+#pragma unroll
+    for (int a = 0; a < NV; ++a) {
+        vel[a] = f.vel(a);
+        q2 = fma(vel[a], vel[a], q2);
+    }
     bool ok = f.ok;
 
     // splitting speed: the largest |u_n| + c over the stencil
@@ -775,10 +854,10 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
         T k = T(0);
 #pragma unroll
         for (int a = 0; a < NV; ++a) {
-            Y[1 + a] = fma(-f.vel[a], X[0], X[1 + a]) * f.irb;
-            k = fma(f.vel[a], X[1 + a], k);
+            Y[1 + a] = fma(-vel[a], X[0], X[1 + a]) * f.irb;
+            k = fma(vel[a], X[1 + a], k);
         }
-        Y[E] = f.gm1 * (fma(T(0.5) * f.q2, X[0], X[E]) - k);
+        Y[E] = f.gm1 * (fma(T(0.5) * q2, X[0], X[E]) - k);
     };
     // cell s: U_s and F(U_s)
     T Fs[NC];
@@ -802,7 +881,7 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
         }
         T dV[NC], G[NC], cw[NC], un, cs;
         f.prim_diff(st[j], st[R], dV);
-        ok = prim_pert<T, NC>(f.ref, dV, tb.gamma, f.igm1, G, cw, un, cs) && ok;
+        ok = prim_pert<T, NC>(f.ref, dV, tb.gamma, tb.igm1, G, cw, un, cs) && ok;
         if (j == R + 1) {
 #pragma unroll
             for (int a = 0; a < NC; ++a) B[a] = G[a];
@@ -831,39 +910,14 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
             const int k1 = k0 + 1;
             const float2 lgs = make_float2(f.lrow(k0, JFs), f.lrow(k1, JFs));
             const float2 lvs = make_float2(f.lrow(k0, JUs), f.lrow(k1, JUs));
-            const float2 fcp = mul2(f2(0.5f), fma2(f2(alpha), lvs, lgs));
-            const float2 fcm = mul2(f2(0.5f), fma2(f2(-alpha), lvs, lgs));
             float2 p2[NS], m2[NS];
 #pragma unroll
             for (int j = 0; j < NS; ++j) {
                 p2[j] = make_float2(dp[k0][j], dp[k1][j]);
                 m2[j] = make_float2(dm[k0][j], dm[k1][j]);
             }
-            float2 pfl[S], pfr[S];
-#pragma unroll
-            for (int h = 0; h < S; ++h) {
-                pfl[h] = (h % 2 == 0 && !MEAN) ? mul2(f2(tb.Psum[h]), fcp) : f2(0.0f);
-                pfr[h] = (h % 2 == 0) ? (MEAN ? mul2(f2(-tb.Psum[h]), m2[R + 1]) : mul2(f2(tb.Psum[h]), fcm))
-                                      : f2(0.0f);
-            }
-            float2 numL = f2(0.0f), denL = f2(0.0f), numR = f2(0.0f), denR = f2(0.0f);
-#pragma unroll
-            for (int m = 0; m <= R; ++m) {
-                const float2 xl = beta_weight2<R, NS>(tb, p2, m, pfl);
-                const float2 xr = beta_weight2<R, NS>(tb, m2, m + 1, pfr);
-                float2 sl = mul2(f2(tb.gsl1[m]), fcp), sr = mul2(f2(tb.gsr1[m]), fcm);
-#pragma unroll
-                for (int j = 0; j <= R; ++j) {
-                    if (m + j != R) sl = fma2(f2(tb.gwl[m][j]), p2[m + j], sl);
-                    if (1 + m + j != R) sr = fma2(f2(tb.gwr[m][j]), m2[1 + m + j], sr);
-                }
-                numL = fma2(xl, sl, numL);
-                denL = fma2(f2(tb.gl[m]), xl, denL);
-                numR = fma2(xr, sr, numR);
-                denR = fma2(f2(tb.gr[m]), xr, denR);
-            }
-            const float2 q = fma2(numL, make_float2(Num<float>::rcp(denL.x), Num<float>::rcp(denL.y)),
-                                  mul2(numR, make_float2(Num<float>::rcp(denR.x), Num<float>::rcp(denR.y))));
+            const float2 q = fdf_state<T, R, MEAN>(tb, p2, m2, vmul(0.5f, vfma(alpha, lvs, lgs)),
+                                                   vmul(0.5f, vfma(-alpha, lvs, lgs)));
             dq[k0] = q.x;
             dq[k1] = q.y;
         }
@@ -871,31 +925,8 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
 #pragma unroll
     for (int kk = kScalarFrom; kk < NC; ++kk) {
         const T lgs = f.lrow(kk, JFs), lvs = f.lrow(kk, JUs);
-        const T fcp = T(0.5) * fma(alpha, lvs, lgs), fcm = T(0.5) * fma(-alpha, lvs, lgs);
-        // zero mean: shifts g+_s and g-_s; mean: centres cell s (left) and s+1 (right)
-        T pfl[S], pfr[S];
-#pragma unroll
-        for (int h = 0; h < S; ++h) {
-            pfl[h] = (h % 2 == 0 && !MEAN) ? tb.Psum[h] * fcp : T(0);
-            pfr[h] = (h % 2 == 0) ? (MEAN ? -tb.Psum[h] * dm[kk][R + 1] : tb.Psum[h] * fcm) : T(0);
-        }
-        T numL = T(0), denL = T(0), numR = T(0), denR = T(0);
-#pragma unroll
-        for (int m = 0; m <= R; ++m) {
-            const T xl = beta_weight<T, R, NS>(tb, dp[kk], m, pfl);
-            const T xr = beta_weight<T, R, NS>(tb, dm[kk], m + 1, pfr);
-            T sl = tb.gsl1[m] * fcp, sr = tb.gsr1[m] * fcm;
-#pragma unroll
-            for (int j = 0; j <= R; ++j) {
-                if (m + j != R) sl = fma(tb.gwl[m][j], dp[kk][m + j], sl);
-                if (1 + m + j != R) sr = fma(tb.gwr[m][j], dm[kk][1 + m + j], sr);
-            }
-            numL = fma(xl, sl, numL);
-            denL = fma(tb.gl[m], xl, denL);
-            numR = fma(xr, sr, numR);
-            denR = fma(tb.gr[m], xr, denR);
-        }
-        dq[kk] = fma(numL, Num<T>::rcp(denL), numR * Num<T>::rcp(denR));
+        dq[kk] = fdf_state<T, R, MEAN>(tb, dp[kk], dm[kk], T(0.5) * fma(alpha, lvs, lgs),
+                                       T(0.5) * fma(-alpha, lvs, lgs));
     }
 
     // back-projection A = (dU/dV) R_V dq at the Roe state
@@ -909,10 +940,12 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
     T ke = T(0);
 #pragma unroll
     for (int a = 0; a < NV; ++a) {
-        A[1 + a] = fma(f.vel[a], w[0], f.rbar * w[1 + a]);
-        ke = fma(f.vel[a], w[1 + a], ke);
+        A[1 + a] = fma(vel[a], w[0], f.rbar * w[1 + a]);
+        ke = fma(vel[a], w[1 + a], ke);
     }
-    A[E] = fma(T(0.5) * f.q2, w[0], fma(f.rbar, ke, w[E] * f.igm1));
+    A[E] = fma(T(0.5) * q2, w[0], fma(f.rbar, ke, w[E] * tb.igm1));
+#pragma unroll
+    for (int a = 0; a < NC; ++a) M[a] = A[a] - B[a];
     return ok;
 }
 
@@ -929,33 +962,49 @@ using TablesFor = typename std::conditional<(VAR & kVarAo) != 0, AoFaceTables<T,
 
 template <typename T, int NC, int R, int VAR>
 __device__ __forceinline__ bool face_eval(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                          T (&B)[NC])
+                                          T (&M)[NC])
 {
-    if constexpr ((VAR & kVarFdFlux) != 0) return face_fdf<T, NC, R, (VAR & kVarMean) != 0>(st, tb, A, B);
-    else return face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0>(st, tb, A, B);
+    if constexpr ((VAR & kVarFdFlux) != 0) return face_fdf<T, NC, R, (VAR & kVarMean) != 0>(st, tb, A, M);
+    else return face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0>(st, tb, A, M);
 }
 
 // Weights of the corrected-flux difference: with the face-flux correction
 // f^_{s+1/2} = F + alpha D2F + beta D4F (Eqs. numFlux_cor, FD-ders; alpha = -1/24,
 // beta = 3/640), f^_{i+1/2} - f^_{i-1/2} = sum_{k=-2..2} c_k dF_{i+k} where
 // dF_s = F_{s+1/2} - F_{s-1/2} and c = (beta, alpha-4beta, 1-2alpha+6beta, alpha-4beta, beta).
-template <typename T>
-__device__ __forceinline__ T corrected_divergence(T d0, T d1, T d2, T d3, T d4)
-{
-    constexpr double al = -1.0 / 24.0, be = 3.0 / 640.0;
-    const T c0 = T(be), c1 = T(al - 4.0 * be), c2 = T(1.0 - 2.0 * al + 6.0 * be);
-    return fma(c0, d0 + d4, fma(c1, d1 + d3, c2 * d2));
-}
-
-// Flux difference across a cell from the five face-flux differences around it:
-// corrected in the FD-Prim form; in the FD-Flux form the reconstructed flux is
-// itself the numerical flux (Eq. design), so only the centre one is used.
+// The jumps come doubled from face_rel (A - M), hence the halves; in the FD-Flux form the
+// reconstructed flux is itself the numerical flux (Eq. design) and only the centre jump counts.
 template <typename T, int VAR>
-__device__ __forceinline__ T flux_divergence(T d0, T d1, T d2, T d3, T d4)
-{
-    if constexpr ((VAR & kVarFdFlux) != 0) return d2;
-    else return corrected_divergence<T>(d0, d1, d2, d3, d4);
-}
+struct Divergence {
+    static constexpr bool kPlain = (VAR & kVarFdFlux) != 0;
+    static constexpr double al = -1.0 / 24.0, be = 3.0 / 640.0;
+    static constexpr double c0 = kPlain ? 0.0 : 0.5 * be, c1 = kPlain ? 0.0 : 0.5 * (al - 4.0 * be),
+                            c2 = kPlain ? 1.0 : 0.5 * (1.0 - 2.0 * al + 6.0 * be);
+    // the flux difference across a cell from the five jumps around it
+    static __device__ __forceinline__ T of(const T (&d)[5])
+    {
+        if constexpr (kPlain) return d[2];
+        return fma(T(c0), d[4], fma(T(c1), d[3], fma(T(c2), d[2], fma(T(c1), d[1], T(c0) * d[0]))));
+    }
+    // the same along a march: `a` holds the partial sums of the next four cells (of the same
+    // order of operations); takes the jump across cell s and returns the difference across s-2
+    static __device__ __forceinline__ T march(T (&a)[4], T d)
+    {
+        if constexpr (kPlain) {
+            const T out = a[0];
+            a[0] = a[1];
+            a[1] = d;
+            return out;
+        } else {
+            const T out = fma(T(c0), d, a[0]);
+            a[0] = fma(T(c1), d, a[1]);
+            a[1] = fma(T(c2), d, a[2]);
+            a[2] = fma(T(c1), d, a[3]);
+            a[3] = T(c0) * d;
+            return out;
+        }
+    }
+};
 
 // Index of cell i along a dimension of n cells after the boundary map:
 // periodic wrap or zero-gradient clamp (outflow).  Periodic wrap is a full

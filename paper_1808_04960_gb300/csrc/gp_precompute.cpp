@@ -493,6 +493,53 @@ bool eigen_factors(dd qs, int N, double *P, double *lambda, double *Ph, double *
     return true;
 }
 
+// The triangular factors of K_m(sigma)^-1 in the window's sums and differences (see GpTables).
+bool window_factors(dd qs, int S, GpTables *out)
+{
+    dd K[kMaxBig][kMaxBig], Q[kMaxS][kMaxS];
+    for (int a = 0; a < S; ++a)
+        for (int b = 0; b < S; ++b) K[a][b] = se_entry(qs, 2 * a, 2 * b);
+    const Chol ch = cholesky(K, S);
+    if (!ch.ok) return false;
+    for (int c = 0; c < S; ++c) {
+        dd e[kMaxBig], x[kMaxBig];
+        for (int r = 0; r < S; ++r) e[r] = make(r == c ? 1.0 : 0.0);
+        chol_solve(ch, e, x);
+        for (int r = 0; r < S; ++r) Q[r][c] = x[r];
+    }
+    // coefficient of pair p's sum (sign 1) or difference (sign -1) in the two cells of the pair
+    auto form = [&](int p, int q, double sign) {
+        const int p2 = S - 1 - p, q2 = S - 1 - q;
+        dd v = make(0.0);
+        for (int i = 0; i < (p == p2 ? 1 : 2); ++i)
+            for (int j = 0; j < (q == q2 ? 1 : 2); ++j) {
+                const double ci = p == p2 ? 1.0 : 0.5 * (i ? 1.0 : sign), cj = q == q2 ? 1.0 : 0.5 * (j ? 1.0 : sign);
+                v = add(v, mul_d(Q[i ? p2 : p][j ? q2 : q], ci * cj));
+            }
+        return v;
+    };
+    const dd A = sqrt_dd(form(0, 0, 1.0)), a = sqrt_dd(form(0, 0, -1.0));
+    dd B = make(0.0), D = make(0.0), kb = make(0.0), kd = make(0.0);
+    if (S > 2) {
+        B = div(form(0, 1, 1.0), A);
+        D = sqrt_dd(sub(form(1, 1, 1.0), mul(B, B)));
+    }
+    if (S > 3) {
+        kb = div(form(0, 1, -1.0), a);
+        kd = sqrt_dd(sub(form(1, 1, -1.0), mul(kb, kb)));
+    }
+    const double inner = S == 3 ? 1.0 : 2.0;   // cells that a unit of s_1 spans
+    out->fA = to_d(A);
+    out->fB = to_d(B);
+    out->fD = to_d(D);
+    out->fa = to_d(a);
+    out->fkb = to_d(kb);
+    out->fkd = to_d(kd);
+    out->fpA = to_d(add(mul_d(A, 2.0), mul_d(B, inner)));
+    out->fpD = to_d(mul_d(D, inner));
+    return A.hi > 0.0 && a.hi > 0.0 && (S < 3 || D.hi > 0.0) && (S < 4 || kd.hi > 0.0);
+}
+
 }  // namespace
 
 int gp_precompute(int R, double ell, double sigma, GpTables *out, char *err, std::size_t errlen, int poly, int recon)
@@ -525,14 +572,6 @@ int gp_precompute(int R, double ell, double sigma, GpTables *out, char *err, std
     if (!side_tables(ql, R, -1, out->wr, out->wbig_r, out->gr, &resid_r, nullptr, out->sr1, err, errlen, kind))
         return 2;
     out->cond_estimate = cond;
-    for (int m = 0; m < S; ++m) {
-        for (int j = 0; j < S; ++j) {
-            out->gwl[m * S + j] = out->gl[m] * out->wl[m * S + j];
-            out->gwr[m * S + j] = out->gr[m] * out->wr[m * S + j];
-        }
-        out->gsl1[m] = out->gl[m] * out->sl1[m];
-        out->gsr1[m] = out->gr[m] * out->sr1[m];
-    }
     // double-double carries ~2^-104 relative; demand cond * 2^-104 < 1e-6
     if (cond * 4.93e-32 > 1e-6) {
         std::snprintf(err, errlen, "covariance of R=%d at l/dx=%g has condition ~%.3g, beyond double-double", R, ell,
@@ -540,7 +579,12 @@ int gp_precompute(int R, double ell, double sigma, GpTables *out, char *err, std
         return 2;
     }
     // smoothness-indicator covariance K_m(sigma) on the points 0..R
-    if (!eigen_factors(qs, S, out->P, out->lambda, out->Ph, out->Psum, nullptr, err, errlen)) return 2;
+    double Ph[kMaxS * kMaxS], Psum[kMaxS];
+    if (!eigen_factors(qs, S, out->P, out->lambda, Ph, Psum, nullptr, err, errlen)) return 2;
+    if (!window_factors(qs, S, out)) {
+        std::snprintf(err, errlen, "K_%d(sigma) is not positive definite in double-double", S);
+        return 2;
+    }
     return 0;
 }
 

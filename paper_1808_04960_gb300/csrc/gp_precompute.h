@@ -21,19 +21,14 @@ struct GpTables {
     // smoothness factors P[h][j] = v_h[j] / sqrt(lambda_h) of K_m(sigma), lambda ascending
     double P[kMaxS * kMaxS];
     double lambda[kMaxS];
-    // The same factors in half form, largest eigenvalue first: K_m(sigma) is
-    // symmetric Toeplitz, hence persymmetric, and the SE kernel is totally
-    // positive, so in descending order of lambda the eigenvectors alternate
-    // symmetric (k even: v_j = v_{S-1-j}) and skew (k odd: v_j = -v_{S-1-j}).
-    // Ph[k*S + j], j < (S+1)/2, holds the first half of P for the k-th largest
-    // eigenvalue; the precompute verifies the alternation.
-    double Ph[kMaxS * kMaxS];
-    double Psum[kMaxS];          // sum_j P_kj of each full row, same order as Ph (0 for skew rows)
+    // The same quadratic form in the window's sums s_j = f_j + f_{R-j} (outer first; the middle cell
+    // itself for odd R+1) and differences t_j = f_{R-j} - f_j, each part factored triangularly:
+    //   f^T K_m(sigma)^-1 f = (fA s_0 + fB s_1)^2 + (fD s_1)^2 + (fa t_0 + fkb t_1)^2 + (fkd t_1)^2
+    // (K_m is persymmetric, so sums and differences do not mix), with the row sums fpA, fpD of the
+    // first two forms over the window's cells.
+    double fA, fB, fD, fa, fkb, fkd, fpA, fpD;
     double sl1[kMaxS];           // sum_j wl[m][j] - 1, from the double-double weights
     double sr1[kMaxS];           // sum_j wr[m][j] - 1
-    // the same scaled by the linear weights, for the weighted sum of Eq. weight_sum:
-    // gwl[m][j] = gl[m] wl[m][j], gsl1[m] = gl[m] sl1[m] (and right)
-    double gwl[kMaxS * kMaxS], gwr[kMaxS * kMaxS], gsl1[kMaxS], gsr1[kMaxS];
     double ls_residual;          // ||M gamma - w||_2 of the left-state system
     double cond_estimate;        // rough condition estimate of K(l)
 };

@@ -242,8 +242,8 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
     // per-component arrays: there the aligned register quads of 16-byte loads cost spills.
     constexpr bool VEC = std::is_same<T, float>::value && NC == 4 && !ONE_SITE && (VAR & (kVarFdFlux | kVarAo)) == 0;
     T *ring = smem;                              // [ROWS][NC][STRIDE], or [ROWS][STRIDE][4] (VEC)
-    T *FA = smem + ROWS * NC * STRIDE;           // [NC][NT] (or [NT][4]): x-face A = F_{s+1/2} - F(U_s)
-    T *FB = FA + NC * NT;                        // [NC][NT] (or [NT][4]): x-face B = F(U_{s+1}) - F(U_s)
+    T *FA = smem + ROWS * NC * STRIDE;           // [NC][NT] (or [NT][4]): x-face A (flux relative to cell s)
+    T *FM = FA + NC * NT;                        // [NC][NT] (or [NT][4]): x-face M (relative to cell s+1)
     // offset of component c of element col in the ring row starting at `base`, and of a face flux
     auto ro = [](int base, int col, int c) { return VEC ? base + col * 4 + c : base + c * STRIDE + col; };
     auto fo = [](int t, int c) { return VEC ? t * 4 + c : c * NT + t; };
@@ -323,15 +323,15 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
     cp_async_wait_all();
     __syncthreads();
 
-    // per column: flux jumps dF_{s'} = F_{s'+1/2} - F_{s'-1/2} across the last five rows,
-    // and A, B of the previous y-face
-    T Dy[5][NC], Ap[NC], Bp[NC];
+    // per column: partial sums of the next four rows' corrected y-differences (Divergence::march), the
+    // difference of output row r, and M of the previous y-face
+    using Dv = Divergence<T, VAR>;
+    T acc[NC][4], divy[NC], Mp[NC];
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) Dy[k][c] = T(0);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) Ap[c] = Bp[c] = T(0);
+    for (int c = 0; c < NC; ++c) {
+        acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = T(0);
+        divy[c] = Mp[c] = T(0);
+    }
 
     for (int s = s_begin; s <= s_end; ++s) {
         if (s < s_end) load_row(s + 2 + R);
@@ -375,29 +375,18 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                         const int cc = pass == 0 ? (c == 1 ? 2 : (c == 2 ? 1 : c)) : c;
                         st[q][c] = ring_at(off[q] + cc * STRIDE);
                     }
-                T An[NC], Bn[NC];
-                ok = face_eval<T, NC, R, VAR>(st, tb, An, Bn) && ok;
+                T An[NC], Mn[NC];
+                ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
                 if (pass == 0) {
-                    T Ac[NC], Bc[NC];   // back to natural order
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
-                        const int pc = c == 1 ? 2 : (c == 2 ? 1 : c);
-                        Ac[c] = An[pc];
-                        Bc[c] = Bn[pc];
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) Dy[k][c] = Dy[k + 1][c];
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        Dy[4][c] = Ac[c] - Ap[c] + Bp[c];   // jump across row s (valid once s > s_begin)
-                        Ap[c] = Ac[c];
-                        Bp[c] = Bc[c];
+                        const int pc = c == 1 ? 2 : (c == 2 ? 1 : c);   // back to natural order
+                        divy[c] = Dv::march(acc[c], An[pc] - Mp[c]);    // jump across row s (valid once s > s_begin)
+                        Mp[c] = Mn[pc];
                     }
                 } else {
                     stage_face(FA, tid, An);
-                    stage_face(FB, tid, Bn);
+                    stage_face(FM, tid, Mn);
                 }
             }
         } else {
@@ -418,24 +407,13 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                         for (int c = 0; c < NC; ++c) st[q][c] = ring_at(ro(base, G + tid, c == 1 ? 2 : (c == 2 ? 1 : c)));
                     }
                 }
-                T An[NC], Bn[NC];
-                ok = face_eval<T, NC, R, VAR>(st, tb, An, Bn) && ok;
-                T Ac[NC], Bc[NC];   // back to natural order
+                T An[NC], Mn[NC];
+                ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
-                    const int pc = c == 1 ? 2 : (c == 2 ? 1 : c);
-                    Ac[c] = An[pc];
-                    Bc[c] = Bn[pc];
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) Dy[k][c] = Dy[k + 1][c];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    Dy[4][c] = Ac[c] - Ap[c] + Bp[c];   // jump across row s (valid once s > s_begin)
-                    Ap[c] = Ac[c];
-                    Bp[c] = Bc[c];
+                    const int pc = c == 1 ? 2 : (c == 2 ? 1 : c);   // back to natural order
+                    divy[c] = Dv::march(acc[c], An[pc] - Mp[c]);    // jump across row s (valid once s > s_begin)
+                    Mp[c] = Mn[pc];
                 }
             }
             // ---- x-faces of output row r ----------------------------------
@@ -444,10 +422,10 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                 T st[NS][NC];
 #pragma unroll
                 for (int q = 0; q < NS; ++q) ring_elem(base, tid + q, st[q]);
-                T An[NC], Bn[NC];
-                ok = face_eval<T, NC, R, VAR>(st, tb, An, Bn) && ok;
+                T An[NC], Mn[NC];
+                ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
                 stage_face(FA, tid, An);
-                stage_face(FB, tid, Bn);
+                stage_face(FM, tid, Mn);
             }
         }
         __syncthreads();
@@ -459,22 +437,18 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                 if (a.u0_is_stencil) ring_elem(ubase, G + tid, un4);
             }
             // x-faces t = tid..tid+5 are s' = x-3..x+2 around cell x = x0 + tid; the flux jumps
-            // dF_k = A_{k+1} - A_k + B_k across the five cells around x (VEC: all components
-            // from 16-byte loads, rolling over k; otherwise one component at a time)
+            // dF_k = A_{k+1} - M_k across the five cells around x (VEC: all components from
+            // 16-byte loads; otherwise one component at a time)
             T dxk[VEC ? 5 : 1][NC];
             if constexpr (VEC) {
-                float4 q = *reinterpret_cast<const float4 *>(FA + tid * 4);
-                T prev[NC] = {q.x, q.y, q.z, q.w};
 #pragma unroll
                 for (int k = 0; k < 5; ++k) {
-                    q = *reinterpret_cast<const float4 *>(FA + (tid + k + 1) * 4);
-                    const float4 w = *reinterpret_cast<const float4 *>(FB + (tid + k) * 4);
-                    const T cur[NC] = {q.x, q.y, q.z, q.w}, b[NC] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        dxk[k][c] = cur[c] - prev[c] + b[c];
-                        prev[c] = cur[c];
-                    }
+                    const float4 q = *reinterpret_cast<const float4 *>(FA + (tid + k + 1) * 4);
+                    const float4 m = *reinterpret_cast<const float4 *>(FM + (tid + k) * 4);
+                    dxk[k][0] = q.x - m.x;
+                    dxk[k][1] = q.y - m.y;
+                    dxk[k][2] = q.z - m.z;
+                    dxk[k][3] = q.w - m.w;
                 }
             }
             T res[NC];
@@ -482,12 +456,8 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
             for (int c = 0; c < NC; ++c) {
                 T dx[5];
 #pragma unroll
-                for (int k = 0; k < 5; ++k)
-                    dx[k] = VEC ? dxk[VEC ? k : 0][c]
-                                : FA[fo(tid + k + 1, c)] - FA[fo(tid + k, c)] + FB[fo(tid + k, c)];
-                const T divx = flux_divergence<T, VAR>(dx[0], dx[1], dx[2], dx[3], dx[4]);
-                const T divy = flux_divergence<T, VAR>(Dy[0][c], Dy[1][c], Dy[2][c], Dy[3][c], Dy[4][c]);
-                const T L = -fma(divx, idx[0], divy * idx[1]);
+                for (int k = 0; k < 5; ++k) dx[k] = VEC ? dxk[VEC ? k : 0][c] : FA[fo(tid + k + 1, c)] - FM[fo(tid + k, c)];
+                const T L = -fma(Dv::of(dx), idx[0], divy[c] * idx[1]);
                 if (NC == 5 || a.mode == kModePartial) {
                     if (chk(c * plane + cell, (long)NC * plane, kChkEpiWrite, a.flags)) a.out[c * plane + cell] = L;
                     res[c] = L;
@@ -682,13 +652,13 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
     cp_async_wait_all();
     __syncthreads();
 
-    T Dz[5][NC], Ap[NC], Bp[NC];
+    using Dv = Divergence<T, VAR>;
+    T acc[NC][4], divz[NC], Mp[NC];
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) Dz[k][c] = T(0);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) Ap[c] = Bp[c] = T(0);
+    for (int c = 0; c < NC; ++c) {
+        acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = T(0);
+        divz[c] = Mp[c] = T(0);
+    }
 
     for (int s = s_begin; s <= s_end; ++s) {
         if (s < s_end) load_plane(s + 2 + R);
@@ -719,19 +689,13 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
                 st[q][3] = rowp[2 * NT];
                 st[q][4] = rowp[4 * NT];
             }
-            T An[NC], Bn[NC];
-            ok = face_eval<T, NC, R, VAR>(st, tb, An, Bn) && ok;
-            const T Ac[NC] = {An[0], An[2], An[3], An[1], An[4]};
-            const T Bc[NC] = {Bn[0], Bn[2], Bn[3], Bn[1], Bn[4]};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) Dz[k][c] = Dz[k + 1][c];
+            T An[NC], Mn[NC];
+            ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                Dz[4][c] = Ac[c] - Ap[c] + Bp[c];
-                Ap[c] = Ac[c];
-                Bp[c] = Bc[c];
+                const int pc = c == 0 || c == 4 ? c : (c == 3 ? 1 : c + 1);   // back to natural order
+                divz[c] = Dv::march(acc[c], An[pc] - Mp[c]);
+                Mp[c] = Mn[pc];
             }
         }
         if (out) {
@@ -740,8 +704,7 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
             T res[NC];
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                const T divz = flux_divergence<T, VAR>(Dz[0][c], Dz[1][c], Dz[2][c], Dz[3][c], Dz[4][c]);
-                const T L = fma(-divz, idx[2], pv[c]);
+                const T L = fma(-divz[c], idx[2], pv[c]);
                 const T un = a.u0_is_stencil ? urow[c * NT] : u0[c];
                 res[c] = stage_epilogue<T>(a, c * cs + cell, L, un, din[c], lov[c], dt, NC * cs);
             }
@@ -801,7 +764,7 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *row = reinterpret_cast<T *>(smem_raw);  // [NC][STRIDE]
     T *FA = row + NC * STRIDE;                 // [NC][NT]
-    T *FB = FA + NC * NT;                      // [NC][NT]
+    T *FM = FA + NC * NT;                      // [NC][NT]
     pdl_enter();
     const T dt = a.dt_dev ? (T)(*a.dt_dev) : (T)a.dt;
     const int tid = threadIdx.x;
@@ -829,12 +792,12 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
             for (int q = 0; q < NS; ++q)
 #pragma unroll
                 for (int c = 0; c < NC; ++c) st[q][c] = row[c * STRIDE + tid + q];
-            T An[NC], Bn[NC];
-            ok = face_eval<T, NC, R, VAR>(st, tb, An, Bn) && ok;
+            T An[NC], Mn[NC];
+            ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 FA[c * NT + tid] = An[c];
-                FB[c * NT + tid] = Bn[c];
+                FM[c * NT + tid] = Mn[c];
             }
         }
         __syncthreads();
@@ -843,11 +806,11 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 const T *fa = FA + c * NT + tid;
-                const T *fb = FB + c * NT + tid;
+                const T *fm = FM + c * NT + tid;
                 T dx[5];
 #pragma unroll
-                for (int k = 0; k < 5; ++k) dx[k] = fa[k + 1] - fa[k] + fb[k];
-                const T L = -flux_divergence<T, VAR>(dx[0], dx[1], dx[2], dx[3], dx[4]) * a.idx[0];
+                for (int k = 0; k < 5; ++k) dx[k] = fa[k + 1] - fm[k];
+                const T L = -Divergence<T, VAR>::of(dx) * a.idx[0];
                 const long cell = (long)c * nx + x0 + tid;
                 const bool epi = a.mode != kModeRHS && chk(cell, (long)NC * nx, kChkEpiRead, a.flags);
                 const T u0 = a.u0_is_stencil ? row[c * STRIDE + G + tid] : (epi ? a.U0[cell] : T(0));
