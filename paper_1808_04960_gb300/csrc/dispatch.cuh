@@ -191,6 +191,7 @@ gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
         if (e != cudaSuccess || occ < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
                                                           "stage2d occupancy");
+        occ = std::min(occ, MINB);   // R = 1's three-CTA build needs 126 registers and would fit four times
     }
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
     s.ctas_per_sm = occ;
