@@ -143,7 +143,10 @@ void gpweno_default_opts(gpweno_opts *opts);
  * factors P_h = v_h / sqrt(lambda_h) of K_m(sigma) (Eq. beta-eigen) are
  * computed in double-double arithmetic on the host (Section 4, step 1),
  * rounded to the plan's dtype and kept with the plan.  Allocates a few
- * hundred bytes of device memory on the current device; the plan must be
+ * hundred bytes of device memory on the current device, and for FP64 2D and 3D
+ * plans a workspace for the face fluxes of a band of the grid (at most 32 MiB, or
+ * 24 layers of the slowest dimension where that is more; none above 1 GiB or
+ * if the allocation fails, the steps then run on slower kernels); the plan must be
  * used on that device.  Returns GPWENO_ERR_PRECOMPUTE if the covariance
  * system is too ill-conditioned for double-double. */
 gpweno_status gpweno_plan_create(gpweno_plan *out, int R, double ell_over_dx, const gpweno_dims *dims,
@@ -176,7 +179,8 @@ gpweno_status gpweno_gp_tables(int R, double ell_over_dx, double sigma_over_dx, 
  * they must not overlap. */
 gpweno_status gpweno_rhs(gpweno_plan plan, const void *U, void *dUdt, void *stream);
 
-/* One SSP-RK3 step in place on U (three fused stage launches; plans with an
+/* One SSP-RK3 step in place on U (three fused stage launches, 3D two per stage, FP64 2D
+ * and 3D two per stage and band of the grid; plans with an
  * external side step with gpweno_rk3_stage instead, GPWENO_ERR_ARG here):
  *   U1 = U + dt L(U);  U2 = 3/4 U + 1/4 (U1 + dt L(U1));  U <- 1/3 U + 2/3 (U2 + dt L(U2)),
  * carried in the equivalent increment form D1 = dt L(U), D2 = 1/4 (D1 + dt L(U+D1)),
@@ -333,7 +337,8 @@ int gpweno_batch_info(gpweno_plan batch, int *block, int *ctas_per_sm, int *grid
 /* Schedule of the last 2D stage launch of a (non-batch, 2D) plan: strip width
  * (columns), number of strips, CTAs launched, and the resident CTAs per SM of
  * the kernel build used (FP32 takes a three-CTA build on small grids, four
- * CTAs otherwise; FP64 one).  All zero before the first launch.  Returns
+ * CTAs otherwise; FP64 one).  FP64 face lists: the strips of the update launch, CTAs and
+ * residency of the face launch.  All zero before the first launch.  Returns
  * GPWENO_ERR_ARG for batch plans and 1D or 3D plans. */
 int gpweno_plan_schedule(gpweno_plan plan, int *strip_width, int *strips, int *grid, int *ctas_per_sm);
 

@@ -211,6 +211,14 @@ gpweno_status gpweno_plan_create(gpweno_plan *out, int R, double ell_over_dx, co
         delete p;
         return cuda_fail(e, "gpweno_plan_create");
     }
+    // FP64 face workspace; a plan that cannot have one steps with the marching kernels
+    if (o.dtype == GPWENO_F64 && dims->ndim >= 2) {
+        size_face_workspace_f64(p);
+        if (p->face_ws_bytes && cudaMalloc(&p->face_ws, p->face_ws_bytes) != cudaSuccess) {
+            p->face_ws = nullptr;
+            (void)cudaGetLastError();   // not an error of this call
+        }
+    }
     *out = p;
     return GPWENO_OK;
 }
@@ -219,6 +227,7 @@ gpweno_status gpweno_plan_destroy(gpweno_plan p)
 {
     if (!p) return GPWENO_OK;
     if (p->ws) cudaFree(p->ws);
+    if (p->face_ws) cudaFree(p->face_ws);
     if (p->batch_inst_dev) cudaFree(p->batch_inst_dev);
     if (p->batch_inst_host) cudaFreeHost(p->batch_inst_host);
     if (p->batch_segs_dev) cudaFree(p->batch_segs_dev);
@@ -344,11 +353,13 @@ static StageIO stage_io(int k, void *U, void *D, void *V1, void *V2, void *lo, d
 }
 
 gpweno_status rk3_sequence(gpweno_plan p, void *U, void *D, void *V1, void *V2, void *lo, double dt,
-                           const double *dt_dev, bool want_rate, cudaStream_t st)
+                           const double *dt_dev, bool want_rate, cudaStream_t st, bool no_workspace)
 {
     for (int k = 0; k < 3; ++k) {
         TraceRange tr(stage_range_name(k));
-        gpweno_status s = launch_stage(p, stage_io(k, U, D, V1, V2, lo, dt, dt_dev, want_rate), st);
+        StageIO io = stage_io(k, U, D, V1, V2, lo, dt, dt_dev, want_rate);
+        io.no_workspace = no_workspace;
+        gpweno_status s = launch_stage(p, io, st);
         if (s != GPWENO_OK) return s;
     }
     return GPWENO_OK;

@@ -3,6 +3,7 @@
 #pragma once
 #include <algorithm>
 
+#include "list.cuh"
 #include "plan.h"
 #include "stage.cuh"
 
@@ -207,14 +208,75 @@ gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R
     return GPWENO_OK;
 }
 
+// Band geometry of the face-list stages (list.cuh) for layers [l0, l0 + nb) of the slowest dimension.
+template <typename T>
+FaceBand<T> face_band(const gpweno_plan_s *p, int l0, int nb)
+{
+    FaceBand<T> b;
+    std::memset(&b, 0, sizeof(b));
+    const int nd = p->dims.ndim;
+    b.buf = static_cast<T *>(p->face_ws);
+    b.size = (long)(p->face_ws_bytes / sizeof(T));
+    b.l0 = l0;
+    b.l1 = l0 + nb;
+    long off = 0;
+    for (int d = 0; d < nd; ++d) {
+        const bool slow = d == nd - 1;
+        b.wrap[d] = p->dims.bc_lo[d] == GPWENO_BC_PERIODIC && (!slow || nb == p->dims.n[d]);
+        for (int e = 0; e < 3; ++e) b.ext[d][e] = e == nd - 1 ? nb : (e < nd ? p->dims.n[e] : 1);
+        if (!b.wrap[d]) b.ext[d][d] += 5;
+        b.lo[d] = b.wrap[d] ? 0 : (slow ? l0 - 3 : -3);
+        b.n[d] = (long)b.ext[d][0] * b.ext[d][1] * b.ext[d][2];
+        b.off[d] = off;
+        off += 2 * (nd + 2) * b.n[d];
+    }
+    return b;
+}
+
+// One stage as face and update launches, band by band.
+template <typename T, int R, int NC, int VAR>
+gpweno_status launch_list(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R, VAR> &tb, cudaStream_t st)
+{
+    constexpr int NT = 256;   // one CTA per SM (255 registers)
+    const Schedule s = schedule2d(a.n[0], a.n[1], NT, p->num_sms);
+    a.W = s.W;
+    a.nstrips = s.nstrips;
+    const int layers = a.n[NC - 3];
+    for (int l0 = 0; l0 < layers; l0 += p->face_ws_layers) {
+        const FaceBand<T> b = face_band<T>(p, l0, std::min(p->face_ws_layers, layers - l0));
+        long items = 0;
+        for (int d = 0; d < NC - 2; ++d) items += (b.n[d] + 31) / 32;
+        const int grid = (int)std::min<long>(p->num_sms, items);
+        cudaError_t e = launch_pdl(face_list_kernel<T, NC, R, VAR, NT>, grid, NT, 0, st, a, b, tb);
+        if (e != cudaSuccess) return cuda_fail(e, "face list kernel launch");
+        const long rows = (long)(b.l1 - b.l0) * (NC == 5 ? a.n[1] : 1) * a.nstrips;
+        e = launch_pdl(face_update_kernel<T, NC, VAR, NT>, (int)std::min<long>(rows, 8L * p->num_sms), NT, 0, st, a, b,
+                       (T)p->gamma);
+        if (e != cudaSuccess) return cuda_fail(e, "face update kernel launch");
+        count_launch(2);
+        if (NC == 4) {
+            p->sched = s;
+            p->sched.grid = grid;
+            p->sched.ctas_per_sm = 1;
+        }
+    }
+    return GPWENO_OK;
+}
+
 // VAR: the scheme variant (kVarMean: non-zero-mean smoothness indicators,
 // kVarFdFlux: the FD-Flux form), a compile-time switch so that the default
 // kernels keep their register budget.
 template <typename T, int R, int VAR>
-gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, cudaStream_t st)
+gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_list, cudaStream_t st)
 {
     StageArgs<T> a = a0;
     const TablesFor<T, R, VAR> tb = make_tables_var<T, R, VAR>(p);
+    // FP64 2D and 3D: face lists wherever the plan has their workspace (measurements in list.cuh); the
+    // marching kernels serve plans without one and the allocation-free step
+    if constexpr (std::is_same<T, double>::value) {
+        if (use_list && p->dims.ndim == 3) return launch_list<T, R, 5, VAR>(p, a, tb, st);
+        if (use_list && p->dims.ndim == 2) return launch_list<T, R, 4, VAR>(p, a, tb, st);
+    }
     if (p->dims.ndim == 3) {
         // (1) xy-plane kernel: P = -(div_x/dx + div_y/dy)
         {
@@ -322,18 +384,41 @@ gpweno_status launch_stage_T(gpweno_plan p, const StageIO &io, cudaStream_t st)
     a.dt = io.dt;
     a.dt_dev = io.dt_dev;
     a.rate = io.want_rate ? p->ws : nullptr;
+    const bool use_list = p->face_ws != nullptr && !io.no_workspace;
     switch (p->R) {
     case 1:
         if constexpr ((VAR & kVarAo) != 0) {
             set_error("GP-AO needs R = 2 or 3");
             return GPWENO_ERR_ARG;
         } else {
-            return launch_stage_R<T, 1, VAR>(p, a, st);
+            return launch_stage_R<T, 1, VAR>(p, a, use_list, st);
         }
-    case 2: return launch_stage_R<T, 2, VAR>(p, a, st);
-    case 3: return launch_stage_R<T, 3, VAR>(p, a, st);
+    case 2: return launch_stage_R<T, 2, VAR>(p, a, use_list, st);
+    case 3: return launch_stage_R<T, 3, VAR>(p, a, use_list, st);
     default: set_error("R=%d not compiled", p->R); return GPWENO_ERR_ARG;
     }
+}
+
+// Workspace of the FP64 face-list stages: layers per band and bytes, chosen at plan creation.  A band has at
+// least 24 layers (the five faces that neighbouring bands repeat then cost at most a fifth of one
+// direction) and up to 32 MiB, which keeps its face fluxes in L2; 32 MiB is 256 K cells in 2D, over fifty
+// warps of faces per SM.  Grids whose 24 layers need more than 1 GiB (3D from 420^2 per plane, 2D
+// from 300 K columns) keep the marching kernels.
+inline void size_face_workspace(gpweno_plan_s *p)
+{
+    const int n = p->dims.n[p->dims.ndim - 1];
+    auto bytes = [&](int nb) {
+        const FaceBand<double> b = face_band<double>(p, 0, nb);
+        long e = 0;
+        for (int d = 0; d < p->dims.ndim; ++d) e += 2L * (p->dims.ndim + 2) * b.n[d];
+        return e * (long)sizeof(double);
+    };
+    int nb = std::min(n, 24);
+    if (bytes(nb) > (1L << 30)) return;
+    while (nb < n && bytes(std::min(n, 2 * nb)) <= (32L << 20)) nb = std::min(n, 2 * nb);
+    const int bands = (n + nb - 1) / nb;
+    p->face_ws_layers = (n + bands - 1) / bands;
+    p->face_ws_bytes = (size_t)std::max(bytes(p->face_ws_layers), bytes(nb));
 }
 
 template <typename T>

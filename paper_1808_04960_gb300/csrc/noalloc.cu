@@ -145,5 +145,5 @@ extern "C" gpweno_status gpweno_rk3_step_noalloc(gpweno_plan p, void *U, double 
     // nothing in the array needs to start at zero: each stage overwrites its buffers
     // completely, and no compensation remainder is carried between calls
     return rk3_sequence(p, U, s0, s0 + stride, s0 + 2 * stride, nullptr, dt, nullptr, false,
-                        static_cast<cudaStream_t>(stream));
+                        static_cast<cudaStream_t>(stream), /*no_workspace=*/true);
 }

@@ -31,6 +31,10 @@ struct gpweno_plan_s {
     // device workspace: [0..2] rate maxima (double bits), [3] flags
     unsigned long long *ws = nullptr;
     gpweno::Schedule sched;
+    // FP64 2D and 3D plans: face fluxes of one band of the grid (null: the marching kernels run)
+    void *face_ws = nullptr;
+    size_t face_ws_bytes = 0;
+    int face_ws_layers = 0;                 // layers of the slowest dimension per band
     const void *halo[2] = {nullptr, nullptr};   // halo buffers of external sides (gpweno_set_halo)
     bool is_batch = false;
     // batch-only data
@@ -75,12 +79,13 @@ struct StageIO {
     double dt = 0.0;
     const double *dt_dev = nullptr;
     bool want_rate = false;
+    bool no_workspace = false;   // keep to the kernels that need no workspace of the plan
 };
 
 // The three stage launches of one SSP-RK3 step on caller buffers:
 // D, V1, V2 are state-sized stage buffers; lo is the compensation remainder (or null).
 gpweno_status rk3_sequence(gpweno_plan p, void *U, void *D, void *V1, void *V2, void *lo, double dt,
-                           const double *dt_dev, bool want_rate, cudaStream_t st);
+                           const double *dt_dev, bool want_rate, cudaStream_t st, bool no_workspace = false);
 // Whether the plan has a GPWENO_BC_EXTERNAL side (slab decomposition).
 bool has_external_side(const gpweno_plan_s *p);
 
@@ -102,6 +107,8 @@ gpweno_status launch_stage_f64_var5(gpweno_plan p, const StageIO &io, cudaStream
 // grids with an external (halo) side: kVarSlab = 8
 gpweno_status launch_stage_f32_var8(gpweno_plan p, const StageIO &io, cudaStream_t st);
 gpweno_status launch_stage_f64_var8(gpweno_plan p, const StageIO &io, cudaStream_t st);
+// layers per band and bytes of an FP64 plan's face workspace (zero bytes: none)
+void size_face_workspace_f64(gpweno_plan p);
 gpweno_status launch_max_rate_f32(gpweno_plan p, const void *U, cudaStream_t st);
 gpweno_status launch_max_rate_f64(gpweno_plan p, const void *U, cudaStream_t st);
 gpweno_status launch_batch_stage_f32(gpweno_plan batch, int stage, void *const *U, void *const *scratch,

@@ -21,6 +21,8 @@ gpweno_status launch_stage_f64(gpweno_plan p, const StageIO &io, cudaStream_t st
     }
 }
 
+void size_face_workspace_f64(gpweno_plan p) { size_face_workspace(p); }
+
 gpweno_status launch_max_rate_f64(gpweno_plan p, const void *U, cudaStream_t st)
 {
     return launch_max_rate_T<double>(p, U, st);
