@@ -52,7 +52,8 @@ constexpr size_t batch_smem_bytes()
 }
 
 // 512 (FP32) or 256 (FP64) resident threads per SM at most 128 / 255 registers each
-template <typename T, int NT>
+// VAR: 0, or kVarFlux for FP32 batches with an HLL or HLLC member
+template <typename T, int NT, int VAR = 0>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
     batch_stage_kernel(const BatchInst<T> *__restrict__ inst, const BatchSeg *__restrict__ segs,
                        const int *__restrict__ cta_start, int stage, const double *__restrict__ dt_dev, int *flags,
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *smem = reinterpret_cast<T *>(smem_raw);
     T rmx = T(0), rmy = T(0);
-    bool ok = true;
+    Physical<T> ph;
     // per-segment arguments live in shared memory (filled by thread 0), which
     // keeps them out of the registers the face evaluation needs
     __shared__ StageArgs<T> sa;
@@ -141,13 +142,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
         // code spills less at 255 registers
         constexpr bool kOneSite = sizeof(T) == 8;
         switch (sR) {
-        case 1: stage2d_segment<T, 1, NT, 4, 0, kOneSite>(sa, bt.t1[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ok); break;
-        case 2: stage2d_segment<T, 2, NT, 4, 0, kOneSite>(sa, bt.t2[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ok); break;
-        default: stage2d_segment<T, 3, NT, 4, 0, kOneSite>(sa, bt.t3[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ok); break;
+        case 1: stage2d_segment<T, 1, NT, 4, VAR, kOneSite>(sa, bt.t1[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+        case 2: stage2d_segment<T, 2, NT, 4, VAR, kOneSite>(sa, bt.t2[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+        default: stage2d_segment<T, 3, NT, 4, VAR, kOneSite>(sa, bt.t3[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
         }
         // the segment ends with a barrier, so thread 0 may overwrite the shared arguments
     }
-    if (__any_sync(0xffffffffu, !ok) && (threadIdx.x & 31) == 0) atomicOr(flags, 1);
+    if (__any_sync(0xffffffffu, !ph.good()) && (threadIdx.x & 31) == 0) atomicOr(flags, 1);
 }
 
 }  // namespace gpweno

@@ -106,10 +106,20 @@ inline bool read_tune_cache(const char *path, unsigned long long sig, BatchTiles
     return found;
 }
 
+// The batch kernel of a block size, for batches of local Lax-Friedrichs members only or of any face flux.
 template <typename T, int NT>
-gpweno_status batch_occupancy(int &occ)
+auto batch_kernel(const gpweno_plan_s *b)
 {
     auto kern = batch_stage_kernel<T, NT>;
+    if constexpr (std::is_same<T, float>::value)
+        if (b->batch_riemann) kern = batch_stage_kernel<T, NT, kVarFlux>;
+    return kern;
+}
+
+template <typename T, int NT>
+gpweno_status batch_occupancy(const gpweno_plan_s *b, int &occ)
+{
+    auto kern = batch_kernel<T, NT>(b);
     const size_t smem = batch_smem_bytes<T, NT>();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "batch smem attribute");
@@ -131,6 +141,7 @@ gpweno_status build_batch_T(gpweno_plan b)
     std::memset(&bt, 0, sizeof(bt));
     std::vector<gpweno_plan> reps[4];
     b->member_tab.assign(n, 0);
+    for (const gpweno_plan p : b->members) b->batch_riemann = b->batch_riemann || p->opts.flux_form != 0;
     for (int k = 0; k < n; ++k) {
         gpweno_plan p = b->members[k];
         auto &rv = reps[p->R];
@@ -183,7 +194,7 @@ gpweno_status build_batch_T(gpweno_plan b)
     const int nt = tiles.nt;
     int cps = tiles.cps;
     int occ = 0;
-    gpweno_status s = nt == 128 ? batch_occupancy<T, 128>(occ) : batch_occupancy<T, 256>(occ);
+    gpweno_status s = nt == 128 ? batch_occupancy<T, 128>(b, occ) : batch_occupancy<T, 256>(b, occ);
     if (s != GPWENO_OK) return s;
     if (cps <= 0 || cps > occ) cps = occ;
     b->batch_nt = nt;
@@ -286,16 +297,14 @@ gpweno_status launch_batch_stage_T(gpweno_plan b, int stage, void *const *U, voi
     }
     BatchTables<T> bt;
     std::memcpy(&bt, b->batch_tables.data(), sizeof(bt));
-    const int *flags = reinterpret_cast<const int *>(b->ws + 3);
-    if (b->batch_nt == 128) {
-        batch_stage_kernel<T, 128><<<b->batch_grid, 128, batch_smem_bytes<T, 128>(), st>>>(
-            static_cast<const BatchInst<T> *>(b->batch_inst_dev), static_cast<const BatchSeg *>(b->batch_segs_dev),
-            static_cast<const int *>(b->batch_cta_dev), stage, dt_dev, const_cast<int *>(flags), bt);
-    } else {
-        batch_stage_kernel<T, 256><<<b->batch_grid, 256, batch_smem_bytes<T, 256>(), st>>>(
-            static_cast<const BatchInst<T> *>(b->batch_inst_dev), static_cast<const BatchSeg *>(b->batch_segs_dev),
-            static_cast<const int *>(b->batch_cta_dev), stage, dt_dev, const_cast<int *>(flags), bt);
-    }
+    int *flags = reinterpret_cast<int *>(b->ws + 3);
+    auto launch = [&](auto kern, int nt, size_t smem) {
+        kern<<<b->batch_grid, nt, smem, st>>>(static_cast<const BatchInst<T> *>(b->batch_inst_dev),
+                                              static_cast<const BatchSeg *>(b->batch_segs_dev),
+                                              static_cast<const int *>(b->batch_cta_dev), stage, dt_dev, flags, bt);
+    };
+    if (b->batch_nt == 128) launch(batch_kernel<T, 128>(b), 128, batch_smem_bytes<T, 128>());
+    else launch(batch_kernel<T, 256>(b), 256, batch_smem_bytes<T, 256>());
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "batch kernel launch");
     count_launch(1);

@@ -192,7 +192,7 @@ gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
         if (e != cudaSuccess || occ < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
                                                           "stage2d occupancy");
-        occ = std::min(occ, MINB);   // R = 1's three-CTA build needs 126 registers and would fit four times
+        occ = std::min(occ, MINB);   // R = 1's three-CTA build needs 125 registers and would fit four times
     }
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
     s.ctas_per_sm = occ;
@@ -325,20 +325,20 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
     } else if (p->dims.ndim == 2) {
         constexpr int NT = kNTxy<T>;
         // FP32, default scheme (also with slab halos): the build for three CTAs per SM (more
-        // registers per thread: R = 1/2/3 132/151/163 instead of 121/128/128) is faster where the
-        // four-CTA schedule cannot fill four CTAs per SM (the grid is row-limited), and for
+        // registers per thread: R = 2/3 140/159 instead of 128; R = 1 needs 125 either way) is faster where
+        // the four-CTA schedule cannot fill four CTAs per SM (the grid is row-limited), and for
         // R = 2, whose four-CTA build is register-capped, where it leaves a CTA fewer than
         // kWideRows rows (three CTAs per SM: fewer, taller segments, fewer warm-up rows).
         // Measured on GB300 (same-box A/B, bitwise-identical results): R = 2 x1.10 at 512^2,
-        // x1.05 at 768^2, x1.017 at 1024^2; R = 1 x1.14 and R = 3 x1.076 at 512^2.  Not taken
-        // where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98), R = 1 at 1024^2 (x0.98),
-        // R = 3 at 1024^2 (x0.986).
-        constexpr bool kHasWide = std::is_same<T, float>::value && (VAR == 0 || VAR == kVarSlab);
+        // x1.05 at 768^2, x1.017 at 1024^2; R = 3 x1.10 at 777 x 613, x1.05 at 1024 x 512.  Not taken
+        // where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98), R = 3 at 1024^2 (x0.986), and R = 1
+        // wherever a fourth CTA per SM has rows (right-hand side of 777 x 613 32.0 us, 35.6 with three).
+        constexpr bool kHasWide = std::is_same<T, float>::value && (VAR & ~(kVarSlab | kVarFlux)) == 0;
         if constexpr (kHasWide) {
             const int slots4 = 512 / NT * p->num_sms;
             const Schedule s4 = schedule2d(a.n[0], a.n[1], NT, slots4);
             const long long rows = (long long)s4.nstrips * a.n[1];
-            const bool row_limited = s4.grid < slots4;
+            const bool row_limited = R == 1 ? s4.grid <= 3 * p->num_sms : s4.grid < slots4;
             const bool short_segments = R == 2 && rows < (long long)kWideRows * s4.grid;
             if (row_limited || short_segments) {
                 gpweno_status r = launch_stage2d<T, R, NT, VAR, 3>(p, a, tb, st);
@@ -347,7 +347,7 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
                 return GPWENO_OK;
             }
         }
-        gpweno_status r = launch_stage2d<T, R, NT, VAR, (sizeof(T) == 4 ? 512 : 256) / NT>(p, a, tb, st);
+        gpweno_status r = launch_stage2d<T, R, NT, VAR, kResident<T, R, VAR> / NT>(p, a, tb, st);
         if (r != GPWENO_OK) return r;
     } else {
         constexpr int NT = kNT1D;

@@ -125,6 +125,45 @@ struct Num<double> {
     static __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 };
 
+// Smallest of a and b, NaN if either is one.
+__device__ __forceinline__ float min_nan(float a, float b)
+{
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float min_nan(float a, float b, float c)
+{
+    float r;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Whether all values that have to be positive were.  FP32 keeps the smallest of them (one three-input
+// minimum for two values, NaN sticks) instead of a comparison each: six values per face cost three
+// instructions, 4096^2 step 2460 -> 2400 us without the checks' share.  FP64 tests the bit patterns, in the
+// integer units.
+template <typename T>
+struct Physical;
+template <>
+struct Physical<float> {
+    float least = 1.0f;
+    __device__ __forceinline__ void need(float a) { least = min_nan(least, a); }
+    __device__ __forceinline__ void need(float a, float b) { least = min_nan(least, a, b); }
+    __device__ __forceinline__ bool good() const { return least > 0.0f; }
+};
+template <>
+struct Physical<double> {
+    bool ok = true;
+    __device__ __forceinline__ void need(double a) { ok = ok && Num<double>::positive(a); }
+    __device__ __forceinline__ void need(double a, double b)
+    {
+        need(a);
+        need(b);
+    }
+    __device__ __forceinline__ bool good() const { return ok; }
+};
+
 // Weight tables of one plan in the arithmetic type.  Passed by value as a
 // kernel parameter so every (warp-uniform) table read is a constant-bank
 // operand.
@@ -176,11 +215,11 @@ struct PrimRef {
 //   k   = rho|u|^2 - rho_s|u_s|^2 = sum_a (g_a u_a + rho_s u_s,a w_a)
 //   E'  = w_p/(gamma-1) + k/2
 //   G   = (g_n,  g_n u_n + m_s,n w_n + w_p,  g_n u_t + m_s,n w_t,  w_n (E+p)_s + u_n (E' + w_p)).
-// Returns false if rho <= 0 or p <= 0 (or NaN); un and cs are the normal velocity and
+// Requires rho > 0 and p > 0 in `ph`; un and cs are the normal velocity and
 // the sound speed of the full state.
 template <typename T, int NC>
-__device__ __forceinline__ bool prim_pert(const PrimRef<T, NC> &r, const T (&w)[NC], T gam, T igm1, T (&G)[NC],
-                                          T (&cw)[NC], T &un, T &cs)
+__device__ __forceinline__ void prim_pert(const PrimRef<T, NC> &r, const T (&w)[NC], T gam, T igm1, T (&G)[NC],
+                                          T (&cw)[NC], T &un, T &cs, Physical<T> &ph)
 {
     constexpr int NV = NC - 2, E = NC - 1;
     const T rho = r.rho + w[0];
@@ -205,7 +244,7 @@ __device__ __forceinline__ bool prim_pert(const PrimRef<T, NC> &r, const T (&w)[
     const T pr = r.p + w[E];
     un = u[0];
     cs = Num<T>::sqrt(Num<T>::pmax(gam * pr * Num<T>::rcp(rho), T(1e-30)));
-    return Num<T>::positive(rho) && Num<T>::positive(pr);
+    ph.need(rho, pr);
 }
 
 // Roe average of the two cells sharing a face (normal-first conserved uL =
@@ -217,7 +256,8 @@ __device__ __forceinline__ bool prim_pert(const PrimRef<T, NC> &r, const T (&w)[
 // With the weight th = sqrt(rho_R) / (sqrt(rho_L) + sqrt(rho_R)) of cell s+1 the Roe velocity is
 // u_s + th du and the Roe enthalpy's sound speed is
 //   c^2 = c_L^2 + th (c_R^2 - c_L^2) + (gamma-1)/2 th (1-th) |du|^2,
-// which needs no enthalpy and only the difference du.
+// which needs no enthalpy and only the difference du.  A density <= 0 of either cell makes c^2 NaN or
+// -infinity (its reciprocal square root is NaN or infinite), so c^2 > 0 checks the densities too.
 template <typename T, int NC>
 struct FaceRoe {
     static constexpr int NV = NC - 2, E = NC - 1;
@@ -229,7 +269,6 @@ struct FaceRoe {
     PrimRef<T, NC> ref;
     T Vs[NC];         // primitive state of cell s
     T dVn[NC];        // V_{s+1} - V_s
-    bool ok;          // rho_L, rho_R, c^2 > 0
 
     // row kk of L_V applied to a primitive vector
     __device__ __forceinline__ T lrow(int kk, const T *v) const
@@ -296,7 +335,6 @@ __device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&
     for (int a = 0; a < NV; ++a) du2 = fma(f.dVn[1 + a], f.dVn[1 + a], du2);
     const T cL2 = tb.gamma * irL * f.ref.p, cR2 = tb.gamma * irR * (f.ref.p + f.dVn[E]);
     f.c2 = fma(tb.hgm1 * fma(-f.th, f.th, f.th), du2, fma(f.th, cR2 - cL2, cL2));
-    f.ok = Num<T>::positive(rL) && Num<T>::positive(rR) && Num<T>::positive(f.c2);
     f.ic = Num<T>::rsqrt(Num<T>::pmax(f.c2, T(1e-30)));
     f.c = f.c2 * f.ic;
     f.rbar = sL * sR;
@@ -608,20 +646,20 @@ __device__ __forceinline__ T ao_side(const AoFaceTables<T, R> &ta, const T (&d)[
 //   * the left state is V_s + R (q_L - L V_s) and the right state
 //     V_{s+1} + R (q_R - L V_{s+1}), using R L = I and sum_m omega_m = 1;
 //   * fluxes and conserved states are perturbations about V_s (prim_pert).
-// Returns false on a non-physical Roe, left, right or neighbour state.
+// Requires a physical Roe, left, right and neighbour state in `ph`.
 // Bound: instruction issue and the FP32 pipe (FP32), the FP64 pipe (FP64), so the count of
 // arithmetic instructions.  Sharing the candidates of a window between both sides, triangular
 // smoothness forms, the Roe sound speed and the neighbour flux from differences, and doubled fluxes
 // measured per step against the form without them: FP32 1024^2 R = 2 232 -> 205 us, 4096^2
 // 2848 -> 2460 us, 3D 512^3 R = 3 63.1 -> 53.4 ms; FP64 512^2 R = 2 3086 -> 2702 us.
-template <typename T, int NC, int R, bool MEAN = false, bool AO = false>
-__device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                         T (&M)[NC])
+// LF: local Lax-Friedrichs only (tb.flux is not read).
+template <typename T, int NC, int R, bool MEAN = false, bool AO = false, bool LF = false>
+__device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
+                                         T (&M)[NC], Physical<T> &ph)
 {
     constexpr int NS = 2 * R + 2;
     constexpr int E = NC - 1;
     const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
-    bool ok = f.ok;
     const T igm1 = tb.igm1, c = f.c, c2 = f.c2, cr = f.cr;
     const PrimRef<T, NC> &ref = f.ref;
     const T(&dn)[NC] = f.dVn;
@@ -693,8 +731,8 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
 
     // --- face flux relative to F(U_s), and F(U_{s+1}) - F(U_s) ---------------
     T GL[NC], GR[NC], cL[NC], cR[NC], B[NC], uL, uR, aL, aR;
-    ok = prim_pert<T, NC>(ref, wL, tb.gamma, igm1, GL, cL, uL, aL) && ok;
-    ok = prim_pert<T, NC>(ref, wR, tb.gamma, igm1, GR, cR, uR, aR) && ok;
+    prim_pert<T, NC>(ref, wL, tb.gamma, igm1, GL, cL, uL, aL, ph);
+    prim_pert<T, NC>(ref, wR, tb.gamma, igm1, GR, cR, uR, aR, ph);
     // B = F(U_{s+1}) - F(U_s) from the exact conserved difference and the primitive one:
     // (dm_n, u'_n dm_n + m_n du_n + dp, u'_t dm_n + m_n du_t, hp du_n + u'_n (dE + dp)), u' = u_{s+1}
     {
@@ -704,9 +742,9 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
 #pragma unroll
         for (int a = 2; a < E; ++a) B[a] = fma(dm, ref.u[a - 1] + dn[a], ref.mn * dn[a]);
         B[E] = fma(dn[1], ref.hp, un * ((st[R + 1][E] - st[R][E]) + dn[E]));
-        ok = ok && Num<T>::positive(ref.p + dn[E]);
+        ph.need(f.c2, ref.p + dn[E]);
     }
-    if (tb.flux == 1) {
+    if (!LF && tb.flux == 1) {
         // HLLC with Einfeldt speeds from the Roe average.  The contact speed enters only
         // through S* - u_K = (dp - rho_K' (S_K' - u_K') du) / D (K' the other side), formed
         // from the small differences dp = p_R - p_L, du = u_R - u_L, so the star states
@@ -746,7 +784,7 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
             else f = fma(SR, dUR[a], GR[a]);
             A[a] = T(2) * f;
         }
-    } else if (tb.flux == 2) {
+    } else if (!LF && tb.flux == 2) {
         // HLL with the same Einfeldt speeds: F_L if S_L >= 0, F_R if S_R <= 0, else
         // (S_R F_L - S_L F_R + S_L S_R (U_R - U_L)) / (S_R - S_L); relative to F(U_s)
         // the flux terms keep that form with G_K = F_K - F(U_s) and c_K = U_K - U_s.
@@ -768,7 +806,6 @@ __device__ __forceinline__ bool face_rel(const T (&st)[2 * R + 2][NC], const Fac
     }
 #pragma unroll
     for (int a = 0; a < NC; ++a) M[a] = fma(T(-2), B[a], A[a]);
-    return ok;
 }
 
 // Sum of the two reconstructed parts of one field (or two) of the FD-Flux form, relative to cell s:
@@ -820,10 +857,10 @@ __device__ __forceinline__ V fdf_state(const FaceTables<T, R> &tb, const V (&p)[
 // with d+-_j = (l(F_j - F_s) +- alpha l(U_j - U_s)) / 2 and g+-_s the cell-s
 // values, each reconstructed part minus g+-_s is
 // sum_m omega_m (w_m . d_m + (sum_j w_mj - 1) g+-_s), and g+_s + g-_s = l(F_s)
-// projects back to F(U_s).  Returns false on a non-physical state.
+// projects back to F(U_s).  Requires physical states in `ph`.
 template <typename T, int NC, int R, bool MEAN = false>
-__device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                         T (&M)[NC])
+__device__ __forceinline__ void face_fdf(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
+                                         T (&M)[NC], Physical<T> &ph)
 {
     constexpr int NS = 2 * R + 2, E = NC - 1, NV = NC - 2;
     const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
@@ -833,7 +870,7 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
         vel[a] = f.vel(a);
         q2 = fma(vel[a], vel[a], q2);
     }
-    bool ok = f.ok;
+    ph.need(f.c2);
 
     // splitting speed: the largest |u_n| + c over the stencil
     T alpha = T(0);
@@ -844,7 +881,7 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
 #pragma unroll
         for (int a = 0; a < NV; ++a) m2 = fma(st[j][1 + a], st[j][1 + a], m2);
         const T pj = f.gm1 * fma(T(-0.5) * m2, ir, st[j][E]);
-        ok = ok && Num<T>::positive(st[j][0]) && Num<T>::positive(pj);
+        ph.need(st[j][0], pj);
         alpha = Num<T>::pmax(alpha, Num<T>::fabs(st[j][1] * ir) +
                                         Num<T>::sqrt(Num<T>::pmax(tb.gamma * pj * ir, T(1e-30))));
     }
@@ -881,7 +918,7 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
         }
         T dV[NC], G[NC], cw[NC], un, cs;
         f.prim_diff(st[j], st[R], dV);
-        ok = prim_pert<T, NC>(f.ref, dV, tb.gamma, tb.igm1, G, cw, un, cs) && ok;
+        prim_pert<T, NC>(f.ref, dV, tb.gamma, tb.igm1, G, cw, un, cs, ph);
         if (j == R + 1) {
 #pragma unroll
             for (int a = 0; a < NC; ++a) B[a] = G[a];
@@ -946,7 +983,6 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
     A[E] = fma(T(0.5) * q2, w[0], fma(f.rbar, ke, w[E] * tb.igm1));
 #pragma unroll
     for (int a = 0; a < NC; ++a) M[a] = A[a] - B[a];
-    return ok;
 }
 
 // Scheme variants chosen at compile time: bit 0 the non-zero-mean smoothness
@@ -954,18 +990,21 @@ __device__ __forceinline__ bool face_fdf(const T (&st)[2 * R + 2][NC], const Fac
 // but a grid with an external (halo) side, whose loaders read ghost layers from
 // halo buffers -- a separate instantiation so that the loaders of the others stay
 // as they are.
-constexpr int kVarMean = 1, kVarFdFlux = 2, kVarAo = 4, kVarSlab = 8;
+// Bit 4 (FP32): HLL and HLLC face fluxes; kernels without it are compiled for the local Lax-Friedrichs
+// flux alone (2 % per step at 1024^2, 3 % in batches, 3-4 % in the GP-AO kernels).  FP64 kernels hold all three.
+constexpr int kVarMean = 1, kVarFdFlux = 2, kVarAo = 4, kVarSlab = 8, kVarFlux = 16;
 
 // Kernel parameter type of a variant's tables.
 template <typename T, int R, int VAR>
 using TablesFor = typename std::conditional<(VAR & kVarAo) != 0, AoFaceTables<T, R>, FaceTables<T, R>>::type;
 
 template <typename T, int NC, int R, int VAR>
-__device__ __forceinline__ bool face_eval(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                          T (&M)[NC])
+__device__ __forceinline__ void face_eval(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
+                                          T (&M)[NC], Physical<T> &ph)
 {
-    if constexpr ((VAR & kVarFdFlux) != 0) return face_fdf<T, NC, R, (VAR & kVarMean) != 0>(st, tb, A, M);
-    else return face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0>(st, tb, A, M);
+    constexpr bool kLf = std::is_same<T, float>::value && (VAR & kVarFlux) == 0;
+    if constexpr ((VAR & kVarFdFlux) != 0) face_fdf<T, NC, R, (VAR & kVarMean) != 0>(st, tb, A, M, ph);
+    else face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0, kLf>(st, tb, A, M, ph);
 }
 
 // Weights of the corrected-flux difference: with the face-flux correction

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(NT, 1) face_list_kernel(StageArgs<T> a, FaceBa
 #pragma unroll
     for (int d = 0; d < ND; ++d) total += items[d] = (fb.n[d] + 31) / 32;
     const long first = total * blockIdx.x / gridDim.x, last = total * (blockIdx.x + 1) / gridDim.x;
-    bool ok = true;
+    Physical<T> ph;
     for (long it = first + warp; it < last; it += NT / 32) {
         int d = 0;
         long f = it;
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(NT, 1) face_list_kernel(StageArgs<T> a, FaceBa
                                : T(0);
         }
         T A[NC], M[NC];
-        ok = face_eval<T, NC, R, VAR>(st, tb, A, M) && ok;
+        face_eval<T, NC, R, VAR>(st, tb, A, M, ph);
         T *dst = fb.buf + fb.off[d] + f;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(NT, 1) face_list_kernel(StageArgs<T> a, FaceBa
             dst[(NC + perm[c]) * fb.n[d]] = M[c];
         }
     }
-    if (__any_sync(0xffffffffu, !ok) && lane == 0) atomicOr(a.flags, 1);
+    if (__any_sync(0xffffffffu, !ph.good()) && lane == 0) atomicOr(a.flags, 1);
 }
 
 // Divergence and stage update of the band's cells: one CTA per strip (at most NT columns) of a row.

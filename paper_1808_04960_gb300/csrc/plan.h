@@ -45,6 +45,7 @@ struct gpweno_plan_s {
     int batch_min_rows = 8;                 // fewest rows of a segment that does not end its strip
     int batch_oversub = 1;                  // CTA shares per resident slot
     int batch_grid = 0;                     // CTAs per launch
+    bool batch_riemann = false;             // some member's face flux is HLL or HLLC
     int batch_nseg = 0;                     // segments in the schedule
     unsigned long long batch_signature = 0; // hash of the instance list (tuning-cache key)
     std::string batch_tune_path;            // tuning cache file (may be empty)
@@ -107,6 +108,12 @@ gpweno_status launch_stage_f64_var5(gpweno_plan p, const StageIO &io, cudaStream
 // grids with an external (halo) side: kVarSlab = 8
 gpweno_status launch_stage_f32_var8(gpweno_plan p, const StageIO &io, cudaStream_t st);
 gpweno_status launch_stage_f64_var8(gpweno_plan p, const StageIO &io, cudaStream_t st);
+// FP32 HLL and HLLC face fluxes: kVarFlux = 16 with the bits above
+gpweno_status launch_stage_f32_var16(gpweno_plan p, const StageIO &io, cudaStream_t st);
+gpweno_status launch_stage_f32_var17(gpweno_plan p, const StageIO &io, cudaStream_t st);
+gpweno_status launch_stage_f32_var20(gpweno_plan p, const StageIO &io, cudaStream_t st);
+gpweno_status launch_stage_f32_var21(gpweno_plan p, const StageIO &io, cudaStream_t st);
+gpweno_status launch_stage_f32_var24(gpweno_plan p, const StageIO &io, cudaStream_t st);
 // layers per band and bytes of an FP64 plan's face workspace (zero bytes: none)
 void size_face_workspace_f64(gpweno_plan p);
 gpweno_status launch_max_rate_f32(gpweno_plan p, const void *U, cudaStream_t st);

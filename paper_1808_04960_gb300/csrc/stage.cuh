@@ -231,7 +231,7 @@ __device__ __forceinline__ void rates2d(const T (&u)[4], T gam, const T (&idx)[3
 // with three radii in one kernel) and in 3D.
 template <typename T, int R, int NT, int NC = 4, int VAR = 0, bool ONE_SITE = false>
 __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const FaceTables<T, R> &tb, int strip, int y0,
-                                                int y1, T *smem, T dt, T &rmx, T &rmy, bool &ok, long zoff = 0)
+                                                int y1, T *smem, T dt, T &rmx, T &rmy, Physical<T> &ph, long zoff = 0)
 {
     using RG = Ring2D<R, NT>;
     constexpr int G = RG::G, ROWS = RG::ROWS, STRIDE = RG::STRIDE;
@@ -376,7 +376,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                         st[q][c] = ring_at(off[q] + cc * STRIDE);
                     }
                 T An[NC], Mn[NC];
-                ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
+                face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
                 if (pass == 0) {
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
@@ -408,7 +408,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                     }
                 }
                 T An[NC], Mn[NC];
-                ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
+                face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     const int pc = c == 1 ? 2 : (c == 2 ? 1 : c);   // back to natural order
@@ -423,7 +423,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
 #pragma unroll
                 for (int q = 0; q < NS; ++q) ring_elem(base, tid + q, st[q]);
                 T An[NC], Mn[NC];
-                ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
+                face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
                 stage_face(FA, tid, An);
                 stage_face(FM, tid, Mn);
             }
@@ -529,10 +529,19 @@ __device__ __forceinline__ long long balanced_start(int b, int grid, long long t
     return total;
 }
 
+// Resident threads per SM the 2D kernel's register budget is cut for: 512 in FP32 (128 registers), 256 in
+// FP64 (255).  GP-AO and FD-Flux faces hold more at once (two stencil sizes, the two split fluxes) and
+// spill there: 384 (168 registers) for R = 1, 2 and 256 for R = 3.  Measured, step on a four-quadrant grid of
+// 1000 x 900: GP-AO R = 3 656 -> 543 us, R = 2 349 -> 340; FD-Flux R = 3 508 -> 412, R = 2 295 -> 281,
+// R = 1 200 -> 195 us; R = 2 with 256 threads loses (430 and 357 us).  The 3D kernels, with one face in
+// flight per thread, need the 512 threads also where they spill (128^3 GP-AO R = 3 2358 us, 2735 with 256).
+template <typename T, int R, int VAR>
+constexpr int kResident = sizeof(T) == 8 ? 256 : ((VAR & (kVarAo | kVarFdFlux)) == 0 ? 512 : (R == 3 ? 256 : 384));
+
 // MINB: resident CTAs per SM the register budget is cut for (the default four 128-thread CTAs
 // in FP32 at 128 registers; three give the compiler ~150 registers, which pays on small grids,
 // see the host's choice in launch_stage_R).
-template <typename T, int R, int NT, int VAR = 0, int MINB = (sizeof(T) == 4 ? 512 : 256) / NT>
+template <typename T, int R, int NT, int VAR = 0, int MINB = kResident<T, R, VAR> / NT>
 __global__ void __launch_bounds__(NT, MINB) stage2d_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -540,7 +549,7 @@ __global__ void __launch_bounds__(NT, MINB) stage2d_kernel(StageArgs<T> a, Table
     pdl_enter();
     const T dt = a.dt_dev ? (T)(*a.dt_dev) : (T)a.dt;
     T rmx = T(0), rmy = T(0);
-    bool ok = true;
+    Physical<T> ph;
     // Persistent schedule: the strips' rows, laid end to end (strip-major),
     // are split into gridDim.x ranges of equal estimated cost; a range that
     // crosses a strip boundary becomes two segments.
@@ -552,10 +561,10 @@ __global__ void __launch_bounds__(NT, MINB) stage2d_kernel(StageArgs<T> a, Table
         const int strip = (int)(u / ny);
         const int y0 = (int)(u - (long long)strip * ny);
         const int y1 = (int)min((long long)ny, y0 + (uend - u));
-        stage2d_segment<T, R, NT, 4, VAR>(a, tb, strip, y0, y1, smem, dt, rmx, rmy, ok);
+        stage2d_segment<T, R, NT, 4, VAR>(a, tb, strip, y0, y1, smem, dt, rmx, rmy, ph);
         u += y1 - y0;
     }
-    finish_block<T>(a, rmx, rmy, T(0), ok);
+    finish_block<T>(a, rmx, rmy, T(0), ph.good());
 }
 
 // ---------------------------------------------------------------------------
@@ -573,7 +582,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT) plane3d
     T *smem = reinterpret_cast<T *>(smem_raw);
     pdl_enter();
     T rmx = T(0), rmy = T(0);
-    bool ok = true;
+    Physical<T> ph;
     const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
     const long per_plane = (long)a.nstrips * ny;
     const long total = per_plane * nz;
@@ -585,10 +594,10 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT) plane3d
         const int strip = (int)(rem / ny);
         const int y0 = (int)(rem - (long)strip * ny);
         const int y1 = (int)min((long long)ny, y0 + (uend - u));
-        stage2d_segment<T, R, NT, 5, VAR, true>(a, tb, strip, y0, y1, smem, T(0), rmx, rmy, ok, (long)z * nx * ny);
+        stage2d_segment<T, R, NT, 5, VAR, true>(a, tb, strip, y0, y1, smem, T(0), rmx, rmy, ph, (long)z * nx * ny);
         u += y1 - y0;
     }
-    if (__any_sync(0xffffffffu, !ok) && (threadIdx.x & 31) == 0) atomicOr(a.flags, 1);
+    if (__any_sync(0xffffffffu, !ph.good()) && (threadIdx.x & 31) == 0) atomicOr(a.flags, 1);
 }
 
 template <int R>
@@ -620,7 +629,7 @@ __device__ __forceinline__ void rates3d(const T (&u)[5], T gam, const T (&idx)[3
 // z-marching over columns [c0, c0+NT) of the flattened xy-plane, planes [z0, z1).
 template <typename T, int R, int NT, int VAR = 0>
 __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const FaceTables<T, R> &tb, long c0, int z0,
-                                               int z1, T *ring, T dt, T (&rm)[3], bool &ok)
+                                               int z1, T *ring, T dt, T (&rm)[3], Physical<T> &ph)
 {
     using RZ = RingZ<R>;
     constexpr int NC = 5, NS = 2 * R + 2;
@@ -690,7 +699,7 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
                 st[q][4] = rowp[4 * NT];
             }
             T An[NC], Mn[NC];
-            ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
+            face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 const int pc = c == 0 || c == 4 ? c : (c == 3 ? 1 : c + 1);   // back to natural order
@@ -729,7 +738,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) stagez_kernel(Stag
     pdl_enter();
     const T dt = a.dt_dev ? (T)(*a.dt_dev) : (T)a.dt;
     T rm[3] = {T(0), T(0), T(0)};
-    bool ok = true;
+    Physical<T> ph;
     const int nz = a.n[2];
     const long plane = (long)a.n[0] * a.n[1];
     const long groups = (plane + NT - 1) / NT;
@@ -740,10 +749,10 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) stagez_kernel(Stag
         const long g = (long)(u / nz);
         const int z0 = (int)(u - (long long)g * nz);
         const int z1 = (int)min((long long)nz, z0 + (uend - u));
-        stagez_segment<T, R, NT, VAR>(a, tb, g * NT, z0, z1, ring, dt, rm, ok);
+        stagez_segment<T, R, NT, VAR>(a, tb, g * NT, z0, z1, ring, dt, rm, ph);
         u += z1 - z0;
     }
-    finish_block<T>(a, rm[0], rm[1], rm[2], ok);
+    finish_block<T>(a, rm[0], rm[1], rm[2], ph.good());
 }
 
 // ---------------------------------------------------------------------------
@@ -770,7 +779,7 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
     const int tid = threadIdx.x;
     const int nx = a.n[0];
     T rmx = T(0);
-    bool ok = true;
+    Physical<T> ph;
     for (int item = blockIdx.x; item < a.nstrips; item += gridDim.x) {
         const int x0 = item * a.W;
         const int Wc = min(a.W, nx - x0);
@@ -793,7 +802,7 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
 #pragma unroll
                 for (int c = 0; c < NC; ++c) st[q][c] = row[c * STRIDE + tid + q];
             T An[NC], Mn[NC];
-            ok = face_eval<T, NC, R, VAR>(st, tb, An, Mn) && ok;
+            face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 FA[c * NT + tid] = An[c];
@@ -828,7 +837,7 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
         }
         __syncthreads();
     }
-    finish_block<T>(a, rmx, T(0), T(0), ok);
+    finish_block<T>(a, rmx, T(0), T(0), ph.good());
 }
 
 // Maximum of (|u_d| + c)/dx_d over all cells (for the CFL time step).
