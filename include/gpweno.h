@@ -337,7 +337,8 @@ int gpweno_batch_info(gpweno_plan batch, int *block, int *ctas_per_sm, int *grid
 /* Schedule of the last 2D stage launch of a (non-batch, 2D) plan: strip width
  * (columns), number of strips, CTAs launched, and the resident CTAs per SM of
  * the kernel build used (FP32 takes a three-CTA build on small grids, four
- * CTAs otherwise; FP64 one).  FP64 face lists: the strips of the update launch, CTAs and
+ * CTAs otherwise; FP64 one).  Small FP32 grids: the tiles' width, tile columns, tiles and residency.
+ * FP64 face lists: the strips of the update launch, CTAs and
  * residency of the face launch.  All zero before the first launch.  Returns
  * GPWENO_ERR_ARG for batch plans and 1D or 3D plans. */
 int gpweno_plan_schedule(gpweno_plan plan, int *strip_width, int *strips, int *grid, int *ctas_per_sm);

@@ -211,6 +211,7 @@ gpweno_status gpweno_plan_create(gpweno_plan *out, int R, double ell_over_dx, co
         delete p;
         return cuda_fail(e, "gpweno_plan_create");
     }
+    if (o.dtype == GPWENO_F32 && dims->ndim == 2) p->tile = choose_tile_f32(p);
     // FP64 face workspace; a plan that cannot have one steps with the marching kernels
     if (o.dtype == GPWENO_F64 && dims->ndim >= 2) {
         size_face_workspace_f64(p);

@@ -6,6 +6,7 @@
 #include "list.cuh"
 #include "plan.h"
 #include "stage.cuh"
+#include "tile.cuh"
 
 namespace gpweno {
 
@@ -151,6 +152,39 @@ inline Schedule schedule2d(int nx, int ny, int nt, int slots)
     s.H = (int)((rows + s.grid - 1) / s.grid);
     s.nseg = 0;
     return s;
+}
+
+constexpr int kNTtile = 256;
+
+// Tiles of a small FP32 2D grid, or none (TX = 0) where strip marching has two CTAs of eight rows per SM:
+// from there on its chain of row iterations is overlapped (512^2 and larger march).  The tile
+// minimises the busiest SM's work and depth: it evaluates `work` warps of faces, at 230 cycles each when
+// its issue slots are full, and a CTA's list is `depth` faces deep, at 1500 cycles each.
+inline Tile2D choose_tile(int nx, int ny, int R, int num_sms)
+{
+    Tile2D best;
+    const int strips = (nx + kNTxy<float> - 6) / (kNTxy<float> - 5);
+    if ((long long)strips * ny / 8 >= 2LL * num_sms) return best;
+    double least = 0.0;
+    for (int TX = 4; TX <= 64; ++TX)
+        for (int TY = 4; TY <= 64; ++TY) {
+            const long G = R + 3;
+            const long elems = (TX + 2 * G) * (TY + 2 * G) + 2 * ((TX + 5L) * TY + TX * (TY + 5L));
+            if (elems * 16 > 100 * 1024) break;   // two CTAs per SM
+            const int tx = (nx + TX - 1) / TX, ty = (ny + TY - 1) / TY;
+            const long tiles = (long)tx * ty, per_sm = (tiles + num_sms - 1) / num_sms;
+            const long warps = ((TX + 5L) * TY + TX * (TY + 5L) + 31) / 32;
+            const long work = per_sm * warps, depth = (per_sm + 1) / 2 * ((warps + kNTtile / 32 - 1) / (kNTtile / 32));
+            const double cost = std::max(230.0 * work, 1500.0 * depth) + 0.2 * std::min(230.0 * work, 1500.0 * depth);
+            if (best.TX == 0 || cost < least) {
+                least = cost;
+                best.TX = TX;
+                best.TY = TY;
+                best.nx = tx;
+                best.ny = ty;
+            }
+        }
+    return best;
 }
 
 template <typename T>
@@ -324,6 +358,25 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
         }
     } else if (p->dims.ndim == 2) {
         constexpr int NT = kNTxy<T>;
+        if constexpr (std::is_same<T, float>::value) {
+            if (p->tile.TX) {
+                auto kern = tile2d_kernel<R, kNTtile, VAR>;
+                const size_t smem = tile2d_elems<R>(p->tile.TX, p->tile.TY) * sizeof(float4);
+                cudaError_t e = cudaSuccess;
+                if (smem > 48 * 1024)
+                    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return cuda_fail(e, "tile2d smem attribute");
+                e = launch_pdl(kern, p->tile.nx * p->tile.ny, kNTtile, smem, st, a, p->tile, tb);
+                if (e != cudaSuccess) return cuda_fail(e, "tile2d kernel launch");
+                p->sched = Schedule();
+                p->sched.W = p->tile.TX;
+                p->sched.nstrips = p->tile.nx;
+                p->sched.grid = p->tile.nx * p->tile.ny;
+                p->sched.ctas_per_sm = kResident<T, R, VAR> / kNTtile;
+                count_launch(1);
+                return GPWENO_OK;
+            }
+        }
         // FP32, default scheme (also with slab halos): the build for three CTAs per SM (more
         // registers per thread: R = 2/3 140/159 instead of 128; R = 1 needs 125 either way) is faster where
         // the four-CTA schedule cannot fill four CTAs per SM (the grid is row-limited), and for

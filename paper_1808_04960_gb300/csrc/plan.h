@@ -10,6 +10,12 @@
 
 namespace gpweno {
 
+// Tiles of the small-grid 2D kernel (tile.cuh); TX = 0: the grid marches.
+struct Tile2D {
+    int TX = 0, TY = 0;   // cells per tile
+    int nx = 0, ny = 0;   // tiles per direction
+};
+
 struct Schedule {
     int W = 0, nstrips = 0, H = 0, nseg = 0, grid = 0;
     int ctas_per_sm = 0;   // resident CTAs per SM of the kernel build the launch used
@@ -31,6 +37,7 @@ struct gpweno_plan_s {
     // device workspace: [0..2] rate maxima (double bits), [3] flags
     unsigned long long *ws = nullptr;
     gpweno::Schedule sched;
+    gpweno::Tile2D tile;                    // FP32 2D plans of small grids
     // FP64 2D and 3D plans: face fluxes of one band of the grid (null: the marching kernels run)
     void *face_ws = nullptr;
     size_t face_ws_bytes = 0;
@@ -114,6 +121,8 @@ gpweno_status launch_stage_f32_var17(gpweno_plan p, const StageIO &io, cudaStrea
 gpweno_status launch_stage_f32_var20(gpweno_plan p, const StageIO &io, cudaStream_t st);
 gpweno_status launch_stage_f32_var21(gpweno_plan p, const StageIO &io, cudaStream_t st);
 gpweno_status launch_stage_f32_var24(gpweno_plan p, const StageIO &io, cudaStream_t st);
+// tiles of an FP32 2D plan (none for larger grids)
+Tile2D choose_tile_f32(const gpweno_plan_s *p);
 // layers per band and bytes of an FP64 plan's face workspace (zero bytes: none)
 void size_face_workspace_f64(gpweno_plan p);
 gpweno_status launch_max_rate_f32(gpweno_plan p, const void *U, cudaStream_t st);

@@ -27,6 +27,11 @@ gpweno_status launch_stage_f32(gpweno_plan p, const StageIO &io, cudaStream_t st
     }
 }
 
+Tile2D choose_tile_f32(const gpweno_plan_s *p)
+{
+    return choose_tile(p->dims.n[0], p->dims.n[1], p->R, p->num_sms);
+}
+
 gpweno_status launch_max_rate_f32(gpweno_plan p, const void *U, cudaStream_t st)
 {
     return launch_max_rate_T<float>(p, U, st);
