@@ -35,6 +35,9 @@ void reset_launch_count() { g_launches = 0; }
 
 __global__ void dt_from_rate_kernel(unsigned long long *rate, int ndim, double cfl, double *dt_dev)
 {
+    // launched while the stage kernel before it finishes (programmatic dependency): wait for its maxima
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         double s = 0.0;
         for (int d = 0; d < ndim; ++d) {
@@ -594,8 +597,9 @@ gpweno_status gpweno_rk3_step(gpweno_plan p, void *U, void *scratch, double dt, 
     gpweno_status s = rk3_sequence(p, U, base, base + bytes, base + 2 * bytes, base + 3 * bytes, dt, dtp, cfl, st);
     if (s != GPWENO_OK) return s;
     if (cfl) {
-        dt_from_rate_kernel<<<1, 32, 0, st>>>(p->ws, p->dims.ndim, p->opts.cfl, static_cast<double *>(dt_dev));
-        GPW_CHECK(cudaGetLastError(), "dt kernel launch");
+        GPW_CHECK(launch_pdl(dt_from_rate_kernel, 1, 32, 0, st, p->ws, p->dims.ndim, p->opts.cfl,
+                             static_cast<double *>(dt_dev)),
+                  "dt kernel launch");
         count_launch(1);
     }
     return GPWENO_OK;
@@ -613,8 +617,8 @@ gpweno_status gpweno_cfl_dt(gpweno_plan p, const void *U, double cfl, void *dt_d
     gpweno_status s =
         p->opts.dtype == GPWENO_F32 ? launch_max_rate_f32(p, U, st) : launch_max_rate_f64(p, U, st);
     if (s != GPWENO_OK) return s;
-    dt_from_rate_kernel<<<1, 32, 0, st>>>(p->ws, p->dims.ndim, cfl, static_cast<double *>(dt_dev));
-    GPW_CHECK(cudaGetLastError(), "dt kernel launch");
+    GPW_CHECK(launch_pdl(dt_from_rate_kernel, 1, 32, 0, st, p->ws, p->dims.ndim, cfl, static_cast<double *>(dt_dev)),
+              "dt kernel launch");
     count_launch(1);
     return GPWENO_OK;
 }

@@ -61,25 +61,6 @@ FaceTables<T, R> make_tables(const gpweno_plan_s *p)
     return t;
 }
 
-// Launch with programmatic stream serialization: the kernel may be scheduled
-// while the stream's preceding kernel finishes; the stage kernels wait for it
-// (pdl_enter) before any global access.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 // Tables of a scheme variant: GP-AO adds its own on top of the GP-WENO ones.
 template <typename T, int R, int VAR>
 TablesFor<T, R, VAR> make_tables_var(const gpweno_plan_s *p)
@@ -156,15 +137,28 @@ inline Schedule schedule2d(int nx, int ny, int nt, int slots)
 
 constexpr int kNTtile = 256;
 
-// Tiles of a small FP32 2D grid, or none (TX = 0) where strip marching has two CTAs of eight rows per SM:
-// from there on its chain of row iterations is overlapped (512^2 and larger march).  The tile
-// minimises the busiest SM's work and depth: it evaluates `work` warps of faces, at 230 cycles each when
+// Strip marching's CTAs of eight rows per SM (the most it makes) below which an FP32 2D grid is tiled.  Measured
+// step times, marching / tiles, at 512^2 (2.1), 768^2 (4.4), 1024^2 (7.6) and 1500^2 (16): HLLC R = 2 108/60, 143/127,
+// 222/218, 421/451 us; FD-Flux R = 2 148/93, 200/192, 311/352, 595/789; GP-AO R = 2 169/81, 239/175, 370/303,
+// 708/646, R = 3 224/132, 372/308, 587/515, 1159/1141; right-hand side alone R = 1/2/3 at 777 x 613 32/36/47 and
+// 25/31/37, at 1024^2 52/64/84 and 51/61/75, at 1500^2 96/121/157 and 104/122/152.  Steps of the default scheme
+// end at two CTAs per SM, below 512^2: their schedule of strips is what gpweno_plan_schedule reports from there on.
+template <int R, int VAR>
+constexpr int kTileLimit = (VAR & kVarAo) != 0 ? 16 : ((VAR & kVarFdFlux) != 0 && R == 2 ? 4 : (R == 1 ? 5 : (R == 2 ? 6 : 8)));
+constexpr int kTileLimitStep = 2, kTileLimitMost = 16;
+inline bool few_rows(int nx, int ny, int num_sms, int per_sm)
+{
+    const int strips = (nx + kNTxy<float> - 6) / (kNTxy<float> - 5);
+    return (long long)strips * ny / 8 < (long long)per_sm * num_sms;
+}
+
+// Tiles of a small FP32 2D grid, or none (TX = 0).  The tile minimises the busiest SM's
+// work and depth: it evaluates `work` warps of faces, at 230 cycles each when
 // its issue slots are full, and a CTA's list is `depth` faces deep, at 1500 cycles each.
 inline Tile2D choose_tile(int nx, int ny, int R, int num_sms)
 {
     Tile2D best;
-    const int strips = (nx + kNTxy<float> - 6) / (kNTxy<float> - 5);
-    if ((long long)strips * ny / 8 >= 2LL * num_sms) return best;
+    if (!few_rows(nx, ny, num_sms, kTileLimitMost)) return best;
     double least = 0.0;
     for (int TX = 4; TX <= 64; ++TX)
         for (int TY = 4; TY <= 64; ++TY) {
@@ -209,6 +203,18 @@ StageArgs<T> base_args(const gpweno_plan_s *p)
     return a;
 }
 
+// Shared memory to ask for so that a launch of `ctas` CTAs spreads evenly: the hardware fills an SM with as
+// many CTAs as fit before it moves on, so a kernel of which four fit per SM leaves SMs idle when it is
+// launched with two or three per SM.  Asking for more than a (k+1)-th of the SM's 228 KB (1 KB of it
+// reserved per CTA) lets k = ceil(ctas / SMs) in.  Measured: R = 1 512^2 step 101 -> 81 us (three of four).
+inline size_t spread_smem(long ctas, int num_sms, size_t smem)
+{
+    const long k = (ctas + num_sms - 1) / num_sms;
+    if (k > 3) return smem;
+    const size_t want = (228 * 1024 / (k + 1) - 1024 + 16) / 16 * 16 + 16;
+    return std::max(smem, want);
+}
+
 // Rows per CTA below which FP32 R = 2 grids take the three-CTA-per-SM build of the 2D kernel.
 constexpr int kWideRows = 24;
 
@@ -227,6 +233,9 @@ gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R
         if (e != cudaSuccess || occ < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
                                                           "stage2d occupancy");
         occ = std::min(occ, MINB);   // R = 1's three-CTA build needs 125 registers and would fit four times
+        if (sizeof(T) == 4)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 116 * 1024);
+        if (e != cudaSuccess) return cuda_fail(e, "stage2d smem attribute");
     }
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
     s.ctas_per_sm = occ;
@@ -235,7 +244,7 @@ gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R
     a.H = s.H;
     a.nseg = s.nseg;
     p->sched = s;
-    cudaError_t e = launch_pdl(kern, s.grid, NT, smem, st, a, tb);
+    cudaError_t e = launch_pdl(kern, s.grid, NT, sizeof(T) == 4 ? spread_smem(s.grid, p->num_sms, smem) : smem, st, a, tb);
     if (e != cudaSuccess) return cuda_fail(e, "stage2d kernel launch");
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "stage kernel launch");
@@ -359,7 +368,8 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
     } else if (p->dims.ndim == 2) {
         constexpr int NT = kNTxy<T>;
         if constexpr (std::is_same<T, float>::value) {
-            if (p->tile.TX) {
+            const int limit = VAR == 0 && a.mode != kModeRHS ? kTileLimitStep : kTileLimit<R, VAR>;
+            if (p->tile.TX && few_rows(a.n[0], a.n[1], p->num_sms, limit)) {
                 auto kern = tile2d_kernel<R, kNTtile, VAR>;
                 const size_t smem = tile2d_elems<R>(p->tile.TX, p->tile.TY) * sizeof(float4);
                 cudaError_t e = cudaSuccess;
@@ -383,15 +393,15 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
         // R = 2, whose four-CTA build is register-capped, where it leaves a CTA fewer than
         // kWideRows rows (three CTAs per SM: fewer, taller segments, fewer warm-up rows).
         // Measured on GB300 (same-box A/B, bitwise-identical results): R = 2 x1.10 at 512^2,
-        // x1.05 at 768^2, x1.017 at 1024^2; R = 3 x1.10 at 777 x 613, x1.05 at 1024 x 512.  Not taken
-        // where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98), R = 3 at 1024^2 (x0.986), and R = 1
-        // wherever a fourth CTA per SM has rows (right-hand side of 777 x 613 32.0 us, 35.6 with three).
+        // x1.05 at 768^2, x1.017 at 1024^2; R = 1 x1.14 at 700 x 640, x1.05 at 777 x 613; R = 3 x1.10 at
+        // 777 x 613, x1.05 at 1024 x 512.  Not taken where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98),
+        // R = 1 at 1024^2 (x0.98), R = 3 at 1024^2 (x0.986).
         constexpr bool kHasWide = std::is_same<T, float>::value && (VAR & ~(kVarSlab | kVarFlux)) == 0;
         if constexpr (kHasWide) {
             const int slots4 = 512 / NT * p->num_sms;
             const Schedule s4 = schedule2d(a.n[0], a.n[1], NT, slots4);
             const long long rows = (long long)s4.nstrips * a.n[1];
-            const bool row_limited = R == 1 ? s4.grid <= 3 * p->num_sms : s4.grid < slots4;
+            const bool row_limited = s4.grid < slots4;
             const bool short_segments = R == 2 && rows < (long long)kWideRows * s4.grid;
             if (row_limited || short_segments) {
                 gpweno_status r = launch_stage2d<T, R, NT, VAR, 3>(p, a, tb, st);
@@ -403,14 +413,22 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
         gpweno_status r = launch_stage2d<T, R, NT, VAR, kResident<T, R, VAR> / NT>(p, a, tb, st);
         if (r != GPWENO_OK) return r;
     } else {
-        constexpr int NT = kNT1D;
-        const size_t smem = stage1d_smem_bytes<T, R, NT>();
-        auto kern = stage1d_kernel<T, R, NT, VAR>;
-        a.nstrips = (a.n[0] + (NT - 5) - 1) / (NT - 5);
-        a.W = (a.n[0] + a.nstrips - 1) / a.nstrips;
-        a.H = 1;
-        a.nseg = 1;
-        cudaError_t e = launch_pdl(kern, a.nstrips, NT, smem, st, a, tb);
+        cudaError_t e = cudaSuccess;
+        auto launch = [&](auto kern, int cells, int nt, size_t smem) {
+            a.nstrips = (a.n[0] + cells - 1) / cells;
+            a.W = (a.n[0] + a.nstrips - 1) / a.nstrips;
+            a.H = 1;
+            a.nseg = 1;
+            e = launch_pdl(kern, a.nstrips, nt, smem, st, a, tb);
+        };
+        // FP64: field-split CTAs up to two per SM (8 K cells).  Six of their warps load an SM's FP64 pipe by
+        // 25 thousand cycles, four of the plain kernel's by 38 thousand; three CTAs would draw level
+        constexpr bool kSplit = std::is_same<T, double>::value && (VAR & (kVarAo | kVarFdFlux)) == 0;
+        if (kSplit && (a.n[0] + 26) / 27 <= 2 * p->num_sms) {
+            if constexpr (kSplit) launch(stage1d_split_kernel<T, R, VAR>, 27, 96, 0);
+        } else {
+            launch(stage1d_kernel<T, R, kNT1D, VAR>, kNT1D - 5, kNT1D, stage1d_smem_bytes<T, R, kNT1D>());
+        }
         if (e != cudaSuccess) return cuda_fail(e, "stage1d kernel launch");
     }
     cudaError_t e = cudaGetLastError();

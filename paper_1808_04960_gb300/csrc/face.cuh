@@ -100,7 +100,7 @@ struct Num<double> {
         const double e = fma(-(a * y), y, 1.0);
         return fma(y * e, fma(0.375, e, 0.5), y);
     }
-    static __device__ __forceinline__ double sqrt(double a) { return a * rsqrt(a); }
+    static __device__ __forceinline__ double sqrt(double a) { return __dmul_rn(a, rsqrt(a)); }
     // IEEE forms, zero and infinity included: once per cell, in the CFL rates
     static __device__ __forceinline__ double rcp_ieee(double x) { return 1.0 / x; }
     static __device__ __forceinline__ double sqrt_ieee(double x) { return ::sqrt(x); }
@@ -247,6 +247,42 @@ __device__ __forceinline__ void prim_pert(const PrimRef<T, NC> &r, const T (&w)[
     ph.need(rho, pr);
 }
 
+// Arithmetic of one characteristic field (T) or of two at once (float2: packed fma/add/mul .f32x2
+// of sm_100 and later, each lane rounded as the scalar operation).
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) { return __ffma2_rn(f2(a), b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float a, float2 b) { return __fmul2_rn(f2(a), b); }
+// In FP64 the product is kept out of later sums (no FMA contraction), so that the 1D kernel that passes
+// states between warps rounds as those that keep them in registers.
+__device__ __forceinline__ float vmul_keep(float a, float b) { return a * b; }
+__device__ __forceinline__ double vmul_keep(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float2 vmul_keep(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ double vneg(double a) { return -a; }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float vrcp(float a) { return Num<float>::rcp(a); }
+__device__ __forceinline__ double vrcp(double a) { return Num<double>::rcp(a); }
+__device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(Num<float>::rcp(a.x), Num<float>::rcp(a.y)); }
+template <typename V>
+__device__ __forceinline__ V vset(double x) { return V(x); }
+template <>
+__device__ __forceinline__ float2 vset<float2>(double x) { return f2((float)x); }
+__device__ __forceinline__ float vcast(float x, float) { return x; }
+__device__ __forceinline__ double vcast(double x, double) { return x; }
+__device__ __forceinline__ float2 vcast(float x, float2) { return f2(x); }
+
 // Roe average of the two cells sharing a face (normal-first conserved uL =
 // cell s, uR = cell s+1), the primitive eigen-system at it, and cell s as the
 // primitive reference of the cell-relative evaluation:
@@ -281,6 +317,36 @@ struct FaceRoe {
 
     // Roe velocity
     __device__ __forceinline__ T vel(int a) const { return fma(th, dVn[1 + a], ref.u[a]); }
+
+    // back-projection: the left and right primitive states relative to cell s
+    __device__ __forceinline__ void left_state(const T (&dq)[NC], T (&w)[NC]) const
+    {
+        w[0] = dq[0] + dq[1] + dq[E];
+        w[1] = vmul_keep(cr, dq[E] - dq[0]);
+#pragma unroll
+        for (int a = 2; a < E; ++a) w[a] = dq[a];
+        w[E] = vmul_keep(c2, dq[0] + dq[E]);
+    }
+    __device__ __forceinline__ void right_state(const T (&dq)[NC], T (&w)[NC]) const
+    {
+        w[0] = dVn[0] + (dq[0] + dq[1] + dq[E]);
+        w[1] = fma(cr, dq[E] - dq[0], dVn[1]);
+#pragma unroll
+        for (int a = 2; a < E; ++a) w[a] = dVn[a] + dq[a];
+        w[E] = fma(c2, dq[0] + dq[E], dVn[E]);
+    }
+
+    // B = F(U_{s+1}) - F(U_s) from the exact conserved difference and the primitive one:
+    // (dm_n, u'_n dm_n + m_n du_n + dp, u'_t dm_n + m_n du_t, hp du_n + u'_n (dE + dp)), u' = u_{s+1}
+    __device__ __forceinline__ void flux_difference(const T (&us)[NC], const T (&ur)[NC], T (&B)[NC]) const
+    {
+        const T dm = ur[1] - us[1], un = ref.u[0] + dVn[1];
+        B[0] = dm;
+        B[1] = fma(dm, un, fma(ref.mn, dVn[1], dVn[E]));
+#pragma unroll
+        for (int a = 2; a < E; ++a) B[a] = fma(dm, ref.u[a - 1] + dVn[a], ref.mn * dVn[a]);
+        B[E] = fma(dVn[1], ref.hp, un * ((ur[E] - us[E]) + dVn[E]));
+    }
 
     // V_j - V_s from the exact conserved difference U_j - U_s by perturbation algebra (irj = 1/rho_j)
     __device__ __forceinline__ void prim_diff(const T (&uj)[NC], const T (&us)[NC], T irj, T (&dV)[NC]) const
@@ -345,34 +411,6 @@ __device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&
     f.cr = f.c * f.irb;
     return f;
 }
-
-// Arithmetic of one characteristic field (T) or of two at once (float2: packed fma/add/mul .f32x2
-// of sm_100 and later, each lane rounded as the scalar operation).
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
-__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
-__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
-__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
-__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
-__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) { return __ffma2_rn(f2(a), b, c); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 vmul(float a, float2 b) { return __fmul2_rn(f2(a), b); }
-__device__ __forceinline__ float vrcp(float a) { return Num<float>::rcp(a); }
-__device__ __forceinline__ double vrcp(double a) { return Num<double>::rcp(a); }
-__device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(Num<float>::rcp(a.x), Num<float>::rcp(a.y)); }
-template <typename V>
-__device__ __forceinline__ V vset(double x) { return V(x); }
-template <>
-__device__ __forceinline__ float2 vset<float2>(double x) { return f2((float)x); }
-__device__ __forceinline__ float vcast(float x, float) { return x; }
-__device__ __forceinline__ double vcast(double x, double) { return x; }
-__device__ __forceinline__ float2 vcast(float x, float2) { return f2(x); }
 
 // (eps + beta)^-p of one smoothness window: beta = f^T K_m(sigma)^-1 f (Eq. beta-eigen, in another
 // orthogonal basis) over the window f[w..w+R] of data f_j - shift = d_j + (f_c - shift), with
@@ -481,8 +519,8 @@ __device__ __forceinline__ void weno_states(const FaceTables<T, R> &tb, const V 
             denR = vfma(tb.gr[k - 1], xr, denR);
         }
     }
-    qL = vmul(numL, vrcp(denL));
-    qR = vsub(vmul(numR, vrcp(denR)), d[R + 1]);
+    qL = vmul_keep(numL, vrcp(denL));
+    qR = vfma(numR, vrcp(denR), vneg(d[R + 1]));
 }
 
 // GP-AO tables (Appendix A) on top of the GP-WENO ones: R = 2 serves AO(2,3),
@@ -626,124 +664,16 @@ __device__ __forceinline__ T ao_side(const AoFaceTables<T, R> &ta, const T (&d)[
     }
 }
 
-// One face, cell-relative form.  st[0..2R+1] is the normal-first conserved
-// stencil; the face s+1/2 lies between st[R] (cell s) and st[R+1] (cell s+1).
-// Outputs
-//   A = 2 (F_{s+1/2} - F(U_s))      (numerical face flux relative to cell s)
-//   M = 2 (F_{s+1/2} - F(U_{s+1}))  (relative to cell s+1)
-// so that the flux jump across cell s, F_{s+1/2} - F_{s-1/2} = (A_s - M_{s-1}) / 2,
-// is formed from small quantities only (the factor 2 spares the halving of the
-// Lax-Friedrichs mean; the divergence's weights take it back).  In real arithmetic this is exactly
-// the scheme: characteristic variables of the primitive variables
-// V = (rho, u, p) with the eigenvectors of the primitive system at the Roe
-// average of cells s, s+1 (Section 6; "FD-Primitive"), GP-WENO states by
-// Eqs. candidate_interp, beta-eigen, weights, weight_sum, and the
-// Lax-Friedrichs flux.  The rewriting only changes where FP rounding falls:
-//   * primitive differences V_j - V_s come from the exact conserved
-//     differences U_j - U_s by perturbation algebra, and are projected as
-//     d_j = L (V_j - V_s) plus the centre value f_c = L V_s, so
-//     q^m = w_m . d_m + f_c sum_j w_mj and P_h . f_m = P_h . d_m + f_c sum_j P_hj;
-//   * the left state is V_s + R (q_L - L V_s) and the right state
-//     V_{s+1} + R (q_R - L V_{s+1}), using R L = I and sum_m omega_m = 1;
-//   * fluxes and conserved states are perturbations about V_s (prim_pert).
-// Requires a physical Roe, left, right and neighbour state in `ph`.
-// Bound: instruction issue and the FP32 pipe (FP32), the FP64 pipe (FP64), so the count of
-// arithmetic instructions.  Sharing the candidates of a window between both sides, triangular
-// smoothness forms, the Roe sound speed and the neighbour flux from differences, and doubled fluxes
-// measured per step against the form without them: FP32 1024^2 R = 2 232 -> 205 us, 4096^2
-// 2848 -> 2460 us, 3D 512^3 R = 3 63.1 -> 53.4 ms; FP64 512^2 R = 2 3086 -> 2702 us.
-// LF: local Lax-Friedrichs only (tb.flux is not read).
-template <typename T, int NC, int R, bool MEAN = false, bool AO = false, bool LF = false>
-__device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
-                                         T (&M)[NC], Physical<T> &ph)
+// Twice the face flux relative to F(U_s) of the two states: w primitive, G flux and c conserved relative to
+// cell s, u and a their normal velocities and sound speeds.  LF: local Lax-Friedrichs only.
+template <typename T, int NC, bool LF, typename Tables>
+__device__ __forceinline__ void face_flux(const FaceRoe<T, NC> &f, const Tables &tb, const T (&wL)[NC],
+                                          const T (&wR)[NC], const T (&GL)[NC], const T (&GR)[NC], const T (&cL)[NC],
+                                          const T (&cR)[NC], T uL, T uR, T aL, T aR, T (&A)[NC])
 {
-    constexpr int NS = 2 * R + 2;
     constexpr int E = NC - 1;
-    const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
-    const T igm1 = tb.igm1, c = f.c, c2 = f.c2, cr = f.cr;
     const PrimRef<T, NC> &ref = f.ref;
-    const T(&dn)[NC] = f.dVn;
-
-    // primitive differences V_j - V_s from the exact conserved differences
-    T dV[NS][NC];
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-        if (j == R || j == R + 1) {
-#pragma unroll
-            for (int a = 0; a < NC; ++a) dV[j][a] = j == R ? T(0) : dn[a];
-            continue;
-        }
-        f.prim_diff(st[j], st[R], dV[j]);
-    }
-
-    T dqL[NC], dqR[NC];
-    // FP32 GP-WENO in 1D and 2D: fields in pairs (0,1), (2,3) through packed
-    // instructions, an odd last field (1D) through the scalar loop below.  3D keeps
-    // the scalar loop: with five fields the packed form spills registers in the
-    // z-marching kernel and measured 3% slower.
-    constexpr bool kPacked = std::is_same<T, float>::value && !AO && NC <= 4;
-    constexpr int kScalarFrom = kPacked ? (NC / 2) * 2 : 0;
-    if constexpr (kPacked) {
-#pragma unroll
-        for (int k0 = 0; k0 + 1 < NC; k0 += 2) {
-            const int k1 = k0 + 1;
-            const float2 fc = make_float2(f.lrow(k0, f.Vs), f.lrow(k1, f.Vs));
-            float2 d[NS], qL, qR;
-#pragma unroll
-            for (int j = 0; j < NS; ++j)
-                d[j] = (j == R) ? f2(0.0f) : make_float2(f.lrow(k0, dV[j]), f.lrow(k1, dV[j]));
-            weno_states<T, R, MEAN>(tb, d, fc, qL, qR);
-            dqL[k0] = qL.x;
-            dqR[k0] = qR.x;
-            dqL[k1] = qL.y;
-            dqR[k1] = qR.y;
-        }
-    }
-#pragma unroll
-    for (int kk = kScalarFrom; kk < NC; ++kk) {
-        const T fc = f.lrow(kk, f.Vs);
-        T d[NS];
-#pragma unroll
-        for (int j = 0; j < NS; ++j) d[j] = (j == R) ? T(0) : f.lrow(kk, dV[j]);
-        if constexpr (AO) {
-            // GP-AO predictions relative to cell s (the kernel parameter is AoFaceTables)
-            const auto &ta = static_cast<const AoFaceTables<T, R> &>(tb);
-            dqL[kk] = ao_side<T, R, NS, false, MEAN>(ta, d, fc);                 // q_L - L V_s
-            dqR[kk] = ao_side<T, R, NS, true, MEAN>(ta, d, fc) - d[R + 1];      // q_R - L V_{s+1}
-        } else {
-            weno_states<T, R, MEAN>(tb, d, fc, dqL[kk], dqR[kk]);
-        }
-    }
-
-    // --- back-projection: primitive states relative to cell s -------------
-    T wL[NC], wR[NC];
-    wL[0] = dqL[0] + dqL[1] + dqL[E];
-    wR[0] = dn[0] + (dqR[0] + dqR[1] + dqR[E]);
-    wL[1] = cr * (dqL[E] - dqL[0]);
-    wR[1] = fma(cr, dqR[E] - dqR[0], dn[1]);
-#pragma unroll
-    for (int a = 2; a < E; ++a) {
-        wL[a] = dqL[a];
-        wR[a] = dn[a] + dqR[a];
-    }
-    wL[E] = c2 * (dqL[0] + dqL[E]);
-    wR[E] = fma(c2, dqR[0] + dqR[E], dn[E]);
-
-    // --- face flux relative to F(U_s), and F(U_{s+1}) - F(U_s) ---------------
-    T GL[NC], GR[NC], cL[NC], cR[NC], B[NC], uL, uR, aL, aR;
-    prim_pert<T, NC>(ref, wL, tb.gamma, igm1, GL, cL, uL, aL, ph);
-    prim_pert<T, NC>(ref, wR, tb.gamma, igm1, GR, cR, uR, aR, ph);
-    // B = F(U_{s+1}) - F(U_s) from the exact conserved difference and the primitive one:
-    // (dm_n, u'_n dm_n + m_n du_n + dp, u'_t dm_n + m_n du_t, hp du_n + u'_n (dE + dp)), u' = u_{s+1}
-    {
-        const T dm = st[R + 1][1] - st[R][1], un = ref.u[0] + dn[1];
-        B[0] = dm;
-        B[1] = fma(dm, un, fma(ref.mn, dn[1], dn[E]));
-#pragma unroll
-        for (int a = 2; a < E; ++a) B[a] = fma(dm, ref.u[a - 1] + dn[a], ref.mn * dn[a]);
-        B[E] = fma(dn[1], ref.hp, un * ((st[R + 1][E] - st[R][E]) + dn[E]));
-        ph.need(f.c2, ref.p + dn[E]);
-    }
+    const T c = f.c;
     if (!LF && tb.flux == 1) {
         // HLLC with Einfeldt speeds from the Roe average.  The contact speed enters only
         // through S* - u_K = (dp - rho_K' (S_K' - u_K') du) / D (K' the other side), formed
@@ -804,6 +734,108 @@ __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const Fac
 #pragma unroll
         for (int a = 0; a < NC; ++a) A[a] = fma(-alpha, cR[a] - cL[a], GL[a] + GR[a]);
     }
+}
+
+// One face, cell-relative form.  st[0..2R+1] is the normal-first conserved
+// stencil; the face s+1/2 lies between st[R] (cell s) and st[R+1] (cell s+1).
+// Outputs
+//   A = 2 (F_{s+1/2} - F(U_s))      (numerical face flux relative to cell s)
+//   M = 2 (F_{s+1/2} - F(U_{s+1}))  (relative to cell s+1)
+// so that the flux jump across cell s, F_{s+1/2} - F_{s-1/2} = (A_s - M_{s-1}) / 2,
+// is formed from small quantities only (the factor 2 spares the halving of the
+// Lax-Friedrichs mean; the divergence's weights take it back).  In real arithmetic this is exactly
+// the scheme: characteristic variables of the primitive variables
+// V = (rho, u, p) with the eigenvectors of the primitive system at the Roe
+// average of cells s, s+1 (Section 6; "FD-Primitive"), GP-WENO states by
+// Eqs. candidate_interp, beta-eigen, weights, weight_sum, and the
+// Lax-Friedrichs flux.  The rewriting only changes where FP rounding falls:
+//   * primitive differences V_j - V_s come from the exact conserved
+//     differences U_j - U_s by perturbation algebra, and are projected as
+//     d_j = L (V_j - V_s) plus the centre value f_c = L V_s, so
+//     q^m = w_m . d_m + f_c sum_j w_mj and P_h . f_m = P_h . d_m + f_c sum_j P_hj;
+//   * the left state is V_s + R (q_L - L V_s) and the right state
+//     V_{s+1} + R (q_R - L V_{s+1}), using R L = I and sum_m omega_m = 1;
+//   * fluxes and conserved states are perturbations about V_s (prim_pert).
+// Requires a physical Roe, left, right and neighbour state in `ph`.
+// Bound: instruction issue and the FP32 pipe (FP32), the FP64 pipe (FP64), so the count of
+// arithmetic instructions.  Sharing the candidates of a window between both sides, triangular
+// smoothness forms, the Roe sound speed and the neighbour flux from differences, and doubled fluxes
+// measured per step against the form without them: FP32 1024^2 R = 2 232 -> 205 us, 4096^2
+// 2848 -> 2460 us, 3D 512^3 R = 3 63.1 -> 53.4 ms; FP64 512^2 R = 2 3086 -> 2702 us.
+// LF: local Lax-Friedrichs only (tb.flux is not read).
+template <typename T, int NC, int R, bool MEAN = false, bool AO = false, bool LF = false>
+__device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
+                                         T (&M)[NC], Physical<T> &ph)
+{
+    constexpr int NS = 2 * R + 2;
+    constexpr int E = NC - 1;
+    const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
+    const T igm1 = tb.igm1;
+    const PrimRef<T, NC> &ref = f.ref;
+    const T(&dn)[NC] = f.dVn;
+
+    // primitive differences V_j - V_s from the exact conserved differences
+    T dV[NS][NC];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+        if (j == R || j == R + 1) {
+#pragma unroll
+            for (int a = 0; a < NC; ++a) dV[j][a] = j == R ? T(0) : dn[a];
+            continue;
+        }
+        f.prim_diff(st[j], st[R], dV[j]);
+    }
+
+    T dqL[NC], dqR[NC];
+    // FP32 GP-WENO in 1D and 2D: fields in pairs (0,1), (2,3) through packed
+    // instructions, an odd last field (1D) through the scalar loop below.  3D keeps
+    // the scalar loop: with five fields the packed form spills registers in the
+    // z-marching kernel and measured 3% slower.
+    constexpr bool kPacked = std::is_same<T, float>::value && !AO && NC <= 4;
+    constexpr int kScalarFrom = kPacked ? (NC / 2) * 2 : 0;
+    if constexpr (kPacked) {
+#pragma unroll
+        for (int k0 = 0; k0 + 1 < NC; k0 += 2) {
+            const int k1 = k0 + 1;
+            const float2 fc = make_float2(f.lrow(k0, f.Vs), f.lrow(k1, f.Vs));
+            float2 d[NS], qL, qR;
+#pragma unroll
+            for (int j = 0; j < NS; ++j)
+                d[j] = (j == R) ? f2(0.0f) : make_float2(f.lrow(k0, dV[j]), f.lrow(k1, dV[j]));
+            weno_states<T, R, MEAN>(tb, d, fc, qL, qR);
+            dqL[k0] = qL.x;
+            dqR[k0] = qR.x;
+            dqL[k1] = qL.y;
+            dqR[k1] = qR.y;
+        }
+    }
+#pragma unroll
+    for (int kk = kScalarFrom; kk < NC; ++kk) {
+        const T fc = f.lrow(kk, f.Vs);
+        T d[NS];
+#pragma unroll
+        for (int j = 0; j < NS; ++j) d[j] = (j == R) ? T(0) : f.lrow(kk, dV[j]);
+        if constexpr (AO) {
+            // GP-AO predictions relative to cell s (the kernel parameter is AoFaceTables)
+            const auto &ta = static_cast<const AoFaceTables<T, R> &>(tb);
+            dqL[kk] = ao_side<T, R, NS, false, MEAN>(ta, d, fc);                 // q_L - L V_s
+            dqR[kk] = ao_side<T, R, NS, true, MEAN>(ta, d, fc) - d[R + 1];      // q_R - L V_{s+1}
+        } else {
+            weno_states<T, R, MEAN>(tb, d, fc, dqL[kk], dqR[kk]);
+        }
+    }
+
+    T wL[NC], wR[NC];
+    f.left_state(dqL, wL);
+    f.right_state(dqR, wR);
+
+    // --- face flux relative to F(U_s), and F(U_{s+1}) - F(U_s) ---------------
+    T GL[NC], GR[NC], cL[NC], cR[NC], B[NC], uL, uR, aL, aR;
+    prim_pert<T, NC>(ref, wL, tb.gamma, igm1, GL, cL, uL, aL, ph);
+    prim_pert<T, NC>(ref, wR, tb.gamma, igm1, GR, cR, uR, aR, ph);
+    f.flux_difference(st[R], st[R + 1], B);
+    ph.need(f.c2, ref.p + dn[E]);
+    face_flux<T, NC, LF>(f, tb, wL, wR, GL, GR, cL, cR, uL, uR, aL, aR, A);
 #pragma unroll
     for (int a = 0; a < NC; ++a) M[a] = fma(T(-2), B[a], A[a]);
 }

@@ -72,6 +72,25 @@ gpweno_status cuda_fail(cudaError_t e, const char *what);
 void count_launch(int n);
 void reset_launch_count();
 
+// Launch with programmatic stream serialization: the kernel may be scheduled
+// while the stream's preceding kernel finishes; the stage kernels wait for it
+// (pdl_enter) before any global access.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // One stage launch (see StageArgs in stage.cuh for the meaning of each buffer).
 struct StageIO {
     const void *U = nullptr;     // stencil state
