@@ -52,11 +52,11 @@ constexpr size_t batch_smem_bytes()
 }
 
 // 512 (FP32) or 256 (FP64) resident threads per SM at most 128 / 255 registers each
-// VAR: 0, or kVarFlux for FP32 batches with an HLL or HLLC member
-template <typename T, int NT, int VAR = 0>
+// VAR: 0, or kVarFlux for FP32 batches with an HLL or HLLC member; SPEC: the stage
+template <typename T, int NT, int VAR, int SPEC>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
     batch_stage_kernel(const BatchInst<T> *__restrict__ inst, const BatchSeg *__restrict__ segs,
-                       const int *__restrict__ cta_start, int stage, const double *__restrict__ dt_dev, int *flags,
+                       const int *__restrict__ cta_start, const double *__restrict__ dt_dev, int *flags,
                        const __grid_constant__ BatchTables<T> bt)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
             a.lo = nullptr;
             a.Dout = nullptr;
             a.Vout = nullptr;
-            if (stage == 0) {
+            if constexpr (SPEC == kSpecFirst) {
                 a.U = I.U;
                 a.Din = nullptr;
                 a.Dout = I.D;
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
                 a.b = T(1);
                 a.mode = kModeIncrement;
                 a.u0_is_stencil = 1;
-            } else if (stage == 1) {
+            } else if constexpr (SPEC == kSpecSecond) {
                 a.U = I.V1;
                 a.Din = I.D;
                 a.Dout = I.D;
@@ -142,9 +142,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
         // code spills less at 255 registers
         constexpr bool kOneSite = sizeof(T) == 8;
         switch (sR) {
-        case 1: stage2d_segment<T, 1, NT, 4, VAR, kOneSite>(sa, bt.t1[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
-        case 2: stage2d_segment<T, 2, NT, 4, VAR, kOneSite>(sa, bt.t2[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
-        default: stage2d_segment<T, 3, NT, 4, VAR, kOneSite>(sa, bt.t3[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+        case 1: stage2d_segment<T, 1, NT, 4, VAR, kOneSite, SPEC>(sa, bt.t1[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+        case 2: stage2d_segment<T, 2, NT, 4, VAR, kOneSite, SPEC>(sa, bt.t2[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+        default: stage2d_segment<T, 3, NT, 4, VAR, kOneSite, SPEC>(sa, bt.t3[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
         }
         // the segment ends with a barrier, so thread 0 may overwrite the shared arguments
     }

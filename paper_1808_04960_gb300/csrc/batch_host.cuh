@@ -106,25 +106,38 @@ inline bool read_tune_cache(const char *path, unsigned long long sig, BatchTiles
     return found;
 }
 
-// The batch kernel of a block size, for batches of local Lax-Friedrichs members only or of any face flux.
-template <typename T, int NT>
+// The batch kernel of a block size and stage, for batches of local Lax-Friedrichs members only or of any face flux.
+template <typename T, int NT, int SPEC>
 auto batch_kernel(const gpweno_plan_s *b)
 {
-    auto kern = batch_stage_kernel<T, NT>;
-    if constexpr (std::is_same<T, float>::value)
-        if (b->batch_riemann) kern = batch_stage_kernel<T, NT, kVarFlux>;
+    auto kern = batch_stage_kernel<T, NT, 0, SPEC>;
+    if constexpr (std::is_same<T, float>::value) {
+        if (b->batch_riemann) kern = batch_stage_kernel<T, NT, kVarFlux, SPEC>;
+    }
     return kern;
+}
+
+template <typename T, int NT>
+auto batch_kernel_of(const gpweno_plan_s *b, int stage)
+{
+    return stage == 0 ? batch_kernel<T, NT, kSpecFirst>(b)
+                      : (stage == 1 ? batch_kernel<T, NT, kSpecSecond>(b) : batch_kernel<T, NT, kSpecFinal>(b));
 }
 
 template <typename T, int NT>
 gpweno_status batch_occupancy(const gpweno_plan_s *b, int &occ)
 {
-    auto kern = batch_kernel<T, NT>(b);
     const size_t smem = batch_smem_bytes<T, NT>();
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "batch smem attribute");
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
-    if (e != cudaSuccess) return cuda_fail(e, "batch occupancy");
+    occ = 1 << 20;
+    for (int stage = 0; stage < 3; ++stage) {   // the schedule serves all three stages
+        auto kern = batch_kernel_of<T, NT>(b, stage);
+        int o = 0;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_fail(e, "batch smem attribute");
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, NT, smem);
+        if (e != cudaSuccess) return cuda_fail(e, "batch occupancy");
+        occ = std::min(occ, o);
+    }
     if (occ < 1) {
         set_error("batch kernel cannot be resident");
         return GPWENO_ERR_CUDA;
@@ -301,10 +314,10 @@ gpweno_status launch_batch_stage_T(gpweno_plan b, int stage, void *const *U, voi
     auto launch = [&](auto kern, int nt, size_t smem) {
         kern<<<b->batch_grid, nt, smem, st>>>(static_cast<const BatchInst<T> *>(b->batch_inst_dev),
                                               static_cast<const BatchSeg *>(b->batch_segs_dev),
-                                              static_cast<const int *>(b->batch_cta_dev), stage, dt_dev, flags, bt);
+                                              static_cast<const int *>(b->batch_cta_dev), dt_dev, flags, bt);
     };
-    if (b->batch_nt == 128) launch(batch_kernel<T, 128>(b), 128, batch_smem_bytes<T, 128>());
-    else launch(batch_kernel<T, 256>(b), 256, batch_smem_bytes<T, 256>());
+    if (b->batch_nt == 128) launch(batch_kernel_of<T, 128>(b, stage), 128, batch_smem_bytes<T, 128>());
+    else launch(batch_kernel_of<T, 256>(b, stage), 256, batch_smem_bytes<T, 256>());
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "batch kernel launch");
     count_launch(1);

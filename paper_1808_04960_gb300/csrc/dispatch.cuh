@@ -220,11 +220,11 @@ constexpr int kWideRows = 24;
 
 // One launch of the 2D stage kernel built for MINB resident CTAs per SM: occupancy (queried
 // once per instantiation), the one-wave schedule, the launch.
-template <typename T, int R, int NT, int VAR, int MINB>
-gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R, VAR> &tb, cudaStream_t st)
+template <typename T, int R, int NT, int VAR, int MINB, int SPEC>
+gpweno_status launch_stage2d_spec(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R, VAR> &tb, cudaStream_t st)
 {
     const size_t smem = stage2d_smem_bytes<T, R, NT>();
-    auto kern = stage2d_kernel<T, R, NT, VAR, MINB>;
+    auto kern = stage2d_kernel<T, R, NT, VAR, MINB, SPEC>;
     static int occ = 0;   // per instantiation: resident CTAs per SM
     if (!occ) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -248,6 +248,46 @@ gpweno_status launch_stage2d(gpweno_plan p, StageArgs<T> a, const TablesFor<T, R
     if (e != cudaSuccess) return cuda_fail(e, "stage2d kernel launch");
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "stage kernel launch");
+    return GPWENO_OK;
+}
+
+// Whether the kernels are compiled for each stage.  FP64 ones are not: their time is the FP64 pipe's.
+template <typename T>
+constexpr bool kPerStage = std::is_same<T, float>::value;
+
+// The same by stage.
+template <typename T, int R, int NT, int VAR, int MINB>
+gpweno_status launch_stage2d(gpweno_plan p, const StageArgs<T> &a, const TablesFor<T, R, VAR> &tb, cudaStream_t st)
+{
+    if constexpr (kPerStage<T>) {
+        if (a.mode == kModeRHS) return launch_stage2d_spec<T, R, NT, VAR, MINB, kSpecRHS>(p, a, tb, st);
+        if (a.mode == kModeFinal) return launch_stage2d_spec<T, R, NT, VAR, MINB, kSpecFinal>(p, a, tb, st);
+        if (a.u0_is_stencil && !a.Din) return launch_stage2d_spec<T, R, NT, VAR, MINB, kSpecFirst>(p, a, tb, st);
+        return launch_stage2d_spec<T, R, NT, VAR, MINB, kSpecSecond>(p, a, tb, st);
+    } else {
+        return launch_stage2d_spec<T, R, NT, VAR, MINB, kSpecAny>(p, a, tb, st);
+    }
+}
+
+// The z-marching launch of a 3D stage: L = P - div_z/dz and the stage update.
+template <typename T, int R, int VAR, int SPEC>
+gpweno_status launch_stagez(gpweno_plan p, const StageArgs<T> &a, const TablesFor<T, R, VAR> &tb, cudaStream_t st)
+{
+    constexpr int NT = kNTz;
+    const size_t smem = stagez_smem_bytes<T, R, NT>();
+    auto kern = stagez_kernel<T, R, NT, VAR, SPEC>;
+    static int occ = 0;
+    if (!occ) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_fail(e, "stagez smem attribute");
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
+        if (e != cudaSuccess || occ < 1)
+            return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "stagez occupancy");
+    }
+    const long long cols = ((long long)a.n[0] * a.n[1] + NT - 1) / NT * a.n[2];
+    const int grid = (int)std::max(1LL, std::min<long long>((long long)occ * p->num_sms, cols / 8));
+    cudaError_t e = launch_pdl(kern, grid, NT, smem, st, a, tb);
+    if (e != cudaSuccess) return cuda_fail(e, "stagez kernel launch");
     return GPWENO_OK;
 }
 
@@ -347,24 +387,17 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             if (e != cudaSuccess) return cuda_fail(e, "plane3d kernel launch");
             count_launch(1);
         }
-        // (2) z-marching kernel: L = P - div_z/dz and the stage update
-        {
-            constexpr int NT = kNTz;
-            const size_t smem = stagez_smem_bytes<T, R, NT>();
-            auto kern = stagez_kernel<T, R, NT, VAR>;
-            static int occ = 0;
-            if (!occ) {
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return cuda_fail(e, "stagez smem attribute");
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
-                if (e != cudaSuccess || occ < 1)
-                    return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "stagez occupancy");
-            }
-            const long long cols = ((long long)a.n[0] * a.n[1] + NT - 1) / NT * a.n[2];
-            const int grid = (int)std::max(1LL, std::min<long long>((long long)occ * p->num_sms, cols / 8));
-            cudaError_t e = launch_pdl(kern, grid, NT, smem, st, a, tb);
-            if (e != cudaSuccess) return cuda_fail(e, "stagez kernel launch");
+        // (2) z-marching kernel
+        gpweno_status r;
+        if constexpr (kPerStage<T>) {
+            if (a.mode == kModeRHS) r = launch_stagez<T, R, VAR, kSpecRHS>(p, a, tb, st);
+            else if (a.mode == kModeFinal) r = launch_stagez<T, R, VAR, kSpecFinal>(p, a, tb, st);
+            else if (a.u0_is_stencil && !a.Din) r = launch_stagez<T, R, VAR, kSpecFirst>(p, a, tb, st);
+            else r = launch_stagez<T, R, VAR, kSpecSecond>(p, a, tb, st);
+        } else {
+            r = launch_stagez<T, R, VAR, kSpecAny>(p, a, tb, st);
         }
+        if (r != GPWENO_OK) return r;
     } else if (p->dims.ndim == 2) {
         constexpr int NT = kNTxy<T>;
         if constexpr (std::is_same<T, float>::value) {

@@ -34,6 +34,13 @@ namespace gpweno {
 // (TwoSum) with a running remainder `lo`, so state rounding does not
 // accumulate over many steps.
 enum StageMode { kModeRHS = 0, kModeIncrement = 1, kModeFinal = 2, kModePartial = 3 };
+// What a stage reads and writes, as a template parameter (SPEC) of the kernels that are compiled per stage:
+// kSpecAny leaves it to StageArgs.  kSpecFirst: increment with U^n = the stencil state and no earlier
+// increment; kSpecSecond: increment on top of an earlier one; kSpecFinal: the last stage; kSpecPartial: kModePartial.
+// The row loop keeps two faces in flight per thread, so each register and instruction beside them counts:
+// without the tests and loads of the other stages R = 2 needs 116-128 registers (128, capped, with them).
+// Measured per step: R = 1/2/3 at 1024^2 164/198/261 -> 142/179/246 us, 4096^2 R = 2 2421 -> 2218 us.
+enum StageSpec { kSpecAny = -1, kSpecRHS = 0, kSpecFirst = 1, kSpecSecond = 2, kSpecFinal = 3, kSpecPartial = 4 };
 // kModePartial (3D only): the xy-plane kernel writes its part of L, -(div_x/dx + div_y/dy),
 // to `out`; the z-marching kernel adds the z part and applies modes 0-2.
 
@@ -182,17 +189,18 @@ __device__ __forceinline__ T two_sum(T a, T b, T &e)
 // Epilogue of one cell and component: L is the RHS, u the stencil-state value of
 // the cell, u0/din/lo the prefetched U^n, previous increment and remainder.
 // Returns the value whose wavespeed the CFL reduction sees (mode 2: U^{n+1}).
-template <typename T>
+template <typename T, int SPEC = kSpecAny>
 __device__ __forceinline__ T stage_epilogue(const StageArgs<T> &a, long cell, T L, T u0, T din, T lo, T dt,
                                             long extent)
 {
     if (!chk(cell, extent, kChkEpiWrite, a.flags)) return L;
-    if (a.mode == kModeRHS) {
+    if (SPEC == kSpecAny ? a.mode == kModeRHS : SPEC == kSpecRHS) {
         a.out[cell] = L;
         return L;
     }
-    const T inc = a.b * fma(dt, L, din);
-    if (a.mode == kModeIncrement) {
+    // uncontracted, so that every kernel adds the same rounded increment
+    const T inc = Num<T>::mul_rn(a.b, fma(dt, L, din));
+    if (SPEC == kSpecAny ? a.mode == kModeIncrement : SPEC != kSpecFinal) {
         a.Dout[cell] = inc;
         a.Vout[cell] = u0 + inc;
         return u0 + inc;
@@ -229,7 +237,7 @@ __device__ __forceinline__ void rates2d(const T (&u)[4], T gam, const T (&idx)[3
 // interleave the two independent faces (faster for the 2D kernels, the FP32 batch
 // included); one copy halves the code, which pays in the FP64 batch (fewer spills
 // with three radii in one kernel) and in 3D.
-template <typename T, int R, int NT, int NC = 4, int VAR = 0, bool ONE_SITE = false>
+template <typename T, int R, int NT, int NC = 4, int VAR = 0, bool ONE_SITE = false, int SPEC = kSpecAny>
 __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const FaceTables<T, R> &tb, int strip, int y0,
                                                 int y1, T *smem, T dt, T &rmx, T &rmy, Physical<T> &ph, long zoff = 0)
 {
@@ -296,13 +304,16 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
             return;
         cp_async_elem(dst, src);
     };
+    // grid columns of this thread's ring elements (the same for every row)
+    const int gx0 = bc_map(x0 - G + min(tid, rowlen - 1), nx, a.per[0]);
+    const int gx1 = bc_map(x0 - G + min(tid + NT, rowlen - 1), nx, a.per[0]);
     auto load_row = [&](int g) {
         T *dst = ring + RG::slot(g) * (NC * STRIDE);
         if ((VAR & kVarSlab) != 0 && NC == 4 && a.slab_dim == 1 && ((g < 0 && a.ext[0]) || (g >= ny && a.ext[1]))) {
             // a ghost row of an external side: from the halo buffer [nc][G][nx]
             const T *src = g < 0 ? a.halo[0] + (long)(g + G) * nx : a.halo[1] + (long)(g - ny) * nx;
             for (int col = tid; col < rowlen; col += NT) {
-                const int gx = bc_map(x0 - G + col, nx, a.per[0]);
+                const int gx = col == tid ? gx0 : gx1;
 #pragma unroll
                 for (int c = 0; c < NC; ++c) stage_copy(dst + ro(0, col, c), src + (long)c * G * nx + gx);
             }
@@ -310,8 +321,9 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
         }
         const int gy = bc_map(g, ny, a.per[1]);
         const T *src = a.U + zoff + (long)gy * nx;
+        static_assert(STRIDE <= 2 * NT, "a ring row is at most two elements per thread");
         for (int col = tid; col < rowlen; col += NT) {
-            const int gx = bc_map(x0 - G + col, nx, a.per[0]);
+            const int gx = col == tid ? gx0 : gx1;
 #pragma unroll
             for (int c = 0; c < NC; ++c) stage_copy(dst + ro(0, col, c), src + c * plane + gx);
         }
@@ -344,13 +356,17 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
         // in flight during the face work
         T u0[NC], din[NC], lov[NC];
         const long cell = zoff + (long)r * nx + x0 + tid;
-        const bool epi = out_row && col_ok && (a.mode == kModeIncrement || a.mode == kModeFinal);
+        constexpr bool kAny = SPEC == kSpecAny;
+        const bool epi = out_row && col_ok && (kAny ? a.mode == kModeIncrement || a.mode == kModeFinal : SPEC != kSpecRHS && SPEC != kSpecPartial);
+        const bool rd_u0 = kAny ? !a.u0_is_stencil : SPEC >= kSpecSecond;
+        const bool rd_din = kAny ? a.Din != nullptr : SPEC >= kSpecSecond;
+        const bool rd_lo = a.lo && (kAny ? a.mode == kModeFinal : SPEC == kSpecFinal);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const bool in = !epi || chk(c * plane + cell, (long)NC * plane, kChkEpiRead, a.flags);
-            u0[c] = (epi && in && !a.u0_is_stencil) ? a.U0[c * plane + cell] : T(0);
-            din[c] = (epi && in && a.Din) ? a.Din[c * plane + cell] : T(0);
-            lov[c] = (epi && in && a.lo && a.mode == kModeFinal) ? a.lo[c * plane + cell] : T(0);
+            u0[c] = (epi && in && rd_u0) ? a.U0[c * plane + cell] : T(0);
+            din[c] = (epi && in && rd_din) ? a.Din[c * plane + cell] : T(0);
+            lov[c] = (epi && in && rd_lo) ? a.lo[c * plane + cell] : T(0);
         }
 
         if constexpr (ONE_SITE) {
@@ -434,7 +450,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
             const int ubase = RG::slot(r) * (NC * STRIDE);
             T un4[NC];
             if constexpr (VEC) {
-                if (a.u0_is_stencil) ring_elem(ubase, G + tid, un4);
+                if (!rd_u0) ring_elem(ubase, G + tid, un4);
             }
             // x-faces t = tid..tid+5 are s' = x-3..x+2 around cell x = x0 + tid; the flux jumps
             // dF_k = A_{k+1} - M_k across the five cells around x (VEC: all components from
@@ -458,15 +474,15 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
 #pragma unroll
                 for (int k = 0; k < 5; ++k) dx[k] = VEC ? dxk[VEC ? k : 0][c] : FA[fo(tid + k + 1, c)] - FM[fo(tid + k, c)];
                 const T L = -fma(Dv::of(dx), idx[0], divy[c] * idx[1]);
-                if (NC == 5 || a.mode == kModePartial) {
+                if (SPEC == kSpecPartial || (kAny && a.mode == kModePartial)) {
                     if (chk(c * plane + cell, (long)NC * plane, kChkEpiWrite, a.flags)) a.out[c * plane + cell] = L;
                     res[c] = L;
                 } else {
-                    const T un = a.u0_is_stencil ? (VEC ? un4[c] : ring_at(ro(ubase, G + tid, c))) : u0[c];
-                    res[c] = stage_epilogue<T>(a, c * plane + cell, L, un, din[c], lov[c], dt, (long)NC * plane);
+                    const T un = !rd_u0 ? (VEC ? un4[c] : ring_at(ro(ubase, G + tid, c))) : u0[c];
+                    res[c] = stage_epilogue<T, SPEC>(a, c * plane + cell, L, un, din[c], lov[c], dt, (long)NC * plane);
                 }
             }
-            if (NC == 4 && a.rate && a.mode == kModeFinal) {
+            if (NC == 4 && a.rate && (kAny ? a.mode == kModeFinal : SPEC == kSpecFinal)) {
                 T rx, ry;
                 rates2d<T>(reinterpret_cast<const T(&)[4]>(res), tb.gamma, idx, rx, ry);
                 rmx = Num<T>::fmax(rmx, rx);
@@ -541,7 +557,7 @@ constexpr int kResident = sizeof(T) == 8 ? 256 : ((VAR & (kVarAo | kVarFdFlux)) 
 // MINB: resident CTAs per SM the register budget is cut for (the default four 128-thread CTAs
 // in FP32 at 128 registers; three give the compiler ~150 registers, which pays on small grids,
 // see the host's choice in launch_stage_R).
-template <typename T, int R, int NT, int VAR = 0, int MINB = kResident<T, R, VAR> / NT>
+template <typename T, int R, int NT, int VAR = 0, int MINB = kResident<T, R, VAR> / NT, int SPEC = kSpecAny>
 __global__ void __launch_bounds__(NT, MINB) stage2d_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -561,7 +577,7 @@ __global__ void __launch_bounds__(NT, MINB) stage2d_kernel(StageArgs<T> a, Table
         const int strip = (int)(u / ny);
         const int y0 = (int)(u - (long long)strip * ny);
         const int y1 = (int)min((long long)ny, y0 + (uend - u));
-        stage2d_segment<T, R, NT, 4, VAR>(a, tb, strip, y0, y1, smem, dt, rmx, rmy, ph);
+        stage2d_segment<T, R, NT, 4, VAR, false, SPEC>(a, tb, strip, y0, y1, smem, dt, rmx, rmy, ph);
         u += y1 - y0;
     }
     finish_block<T>(a, rmx, rmy, T(0), ph.good());
@@ -594,7 +610,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT) plane3d
         const int strip = (int)(rem / ny);
         const int y0 = (int)(rem - (long)strip * ny);
         const int y1 = (int)min((long long)ny, y0 + (uend - u));
-        stage2d_segment<T, R, NT, 5, VAR, true>(a, tb, strip, y0, y1, smem, T(0), rmx, rmy, ph, (long)z * nx * ny);
+        stage2d_segment<T, R, NT, 5, VAR, true, kSpecPartial>(a, tb, strip, y0, y1, smem, T(0), rmx, rmy, ph, (long)z * nx * ny);
         u += y1 - y0;
     }
     if (__any_sync(0xffffffffu, !ph.good()) && (threadIdx.x & 31) == 0) atomicOr(a.flags, 1);
@@ -627,7 +643,7 @@ __device__ __forceinline__ void rates3d(const T (&u)[5], T gam, const T (&idx)[3
 }
 
 // z-marching over columns [c0, c0+NT) of the flattened xy-plane, planes [z0, z1).
-template <typename T, int R, int NT, int VAR = 0>
+template <typename T, int R, int NT, int VAR = 0, int SPEC = kSpecAny>
 __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const FaceTables<T, R> &tb, long c0, int z0,
                                                int z1, T *ring, T dt, T (&rm)[3], Physical<T> &ph)
 {
@@ -676,14 +692,18 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
         const bool out = r >= z0 && col_ok;
         const long cell = (long)r * plane + col;
         T pv[NC], u0[NC], din[NC], lov[NC];
-        const bool epi = out && (a.mode == kModeIncrement || a.mode == kModeFinal);
+        constexpr bool kAny = SPEC == kSpecAny;
+        const bool epi = out && (kAny ? a.mode == kModeIncrement || a.mode == kModeFinal : SPEC != kSpecRHS);
+        const bool rd_u0 = kAny ? !a.u0_is_stencil : SPEC >= kSpecSecond;
+        const bool rd_din = kAny ? a.Din != nullptr : SPEC >= kSpecSecond;
+        const bool rd_lo = a.lo && (kAny ? a.mode == kModeFinal : SPEC == kSpecFinal);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const bool in = !out || chk(c * cs + cell, NC * cs, kChkEpiRead, a.flags);
             pv[c] = (out && in) ? a.P[c * cs + cell] : T(0);
-            u0[c] = (epi && in && !a.u0_is_stencil) ? a.U0[c * cs + cell] : T(0);
-            din[c] = (epi && in && a.Din) ? a.Din[c * cs + cell] : T(0);
-            lov[c] = (epi && in && a.lo && a.mode == kModeFinal) ? a.lo[c * cs + cell] : T(0);
+            u0[c] = (epi && in && rd_u0) ? a.U0[c * cs + cell] : T(0);
+            din[c] = (epi && in && rd_din) ? a.Din[c * cs + cell] : T(0);
+            lov[c] = (epi && in && rd_lo) ? a.lo[c * cs + cell] : T(0);
         }
         if (col_ok) {
             // normal-first for a z-face: (rho, rho w, rho u, rho v, E)
@@ -714,10 +734,10 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 const T L = fma(-divz[c], idx[2], pv[c]);
-                const T un = a.u0_is_stencil ? urow[c * NT] : u0[c];
-                res[c] = stage_epilogue<T>(a, c * cs + cell, L, un, din[c], lov[c], dt, NC * cs);
+                const T un = !rd_u0 ? urow[c * NT] : u0[c];
+                res[c] = stage_epilogue<T, SPEC>(a, c * cs + cell, L, un, din[c], lov[c], dt, NC * cs);
             }
-            if (a.rate && a.mode == kModeFinal) {
+            if (a.rate && (kAny ? a.mode == kModeFinal : SPEC == kSpecFinal)) {
                 T rx, ry, rz;
                 rates3d<T>(res, tb.gamma, idx, rx, ry, rz);
                 rm[0] = Num<T>::fmax(rm[0], rx);
@@ -730,7 +750,7 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
     }
 }
 
-template <typename T, int R, int NT, int VAR = 0>
+template <typename T, int R, int NT, int VAR = 0, int SPEC = kSpecAny>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) stagez_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -749,7 +769,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) stagez_kernel(Stag
         const long g = (long)(u / nz);
         const int z0 = (int)(u - (long long)g * nz);
         const int z1 = (int)min((long long)nz, z0 + (uend - u));
-        stagez_segment<T, R, NT, VAR>(a, tb, g * NT, z0, z1, ring, dt, rm, ph);
+        stagez_segment<T, R, NT, VAR, SPEC>(a, tb, g * NT, z0, z1, ring, dt, rm, ph);
         u += z1 - z0;
     }
     finish_block<T>(a, rm[0], rm[1], rm[2], ph.good());
