@@ -10,8 +10,35 @@
 
 namespace gpweno {
 
-// Block size of the 3D z-marching kernel (contiguous runs of 256 xy-columns).
+// Block size of the 3D z-marching kernel (contiguous runs of 256 xy-columns; FP32 also runs of 128, see launch_stagez).
 constexpr int kNTz = 256;
+// CTAs of a 3D launch that marches `groups` groups (strips of planes, runs of columns) of n layers each, and an
+// estimate of its time in layer iterations.  The layers of all groups, end to end, are cut into equal
+// ranges; a range evaluates five layers of faces before its first, and again where it enters another group.
+// With m ranges per group none does: ceil(n/m) + 5 iterations.  An iteration of an SM with 4 or 8 warps
+// takes the same time (a chain of one thread's instructions), with 12 about 1.2 and with 16 (all that are
+// resident) 1.5 times that.  Taken against the cut into as many ranges of at least eight layers as fit at once
+// (`full`).  Measured steps, R = 3: 32^3 152 -> 103, 56^3 238 -> 160,
+// 64^3 252 -> 215, 80^3 348 -> 342, 96^3 507 -> 424 us.
+struct Cut3D {
+    int grid;
+    double cost;
+};
+inline Cut3D cut3d(long long groups, int n, int occ, int num_sms, int block)
+{
+    auto pace = [&](long long ctas) {
+        const long long warps = std::min<long long>(occ, (ctas + num_sms - 1) / num_sms) * (block / 32);
+        return warps <= 8 ? 1.0 : (warps <= 12 ? 1.2 : 1.5);
+    };
+    const long long slots = (long long)occ * num_sms, total = groups * n;
+    const long long full = std::max(1LL, std::min(slots, total / 8));
+    Cut3D best = {(int)full, ((total + full - 1) / full + (total % full || n % (total / full) ? 10 : 5)) * pace(full)};
+    for (long long m = 1; m <= n && groups * m <= slots; ++m) {
+        const double cost = ((n + m - 1) / m + 5) * pace(groups * m);
+        if (cost < best.cost) best = {(int)(groups * m), cost};
+    }
+    return best;
+}
 // Block size of the xy-sweeping kernels (2D stage, 3D plane).  FP32: 128 threads
 // and four CTAs per SM, with the same 128 registers per thread as two 256-thread
 // CTAs.  A strip is then at most 123 columns, so every warp of a CTA evaluates
@@ -207,6 +234,8 @@ StageArgs<T> base_args(const gpweno_plan_s *p)
 // many CTAs as fit before it moves on, so a kernel of which four fit per SM leaves SMs idle when it is
 // launched with two or three per SM.  Asking for more than a (k+1)-th of the SM's 228 KB (1 KB of it
 // reserved per CTA) lets k = ceil(ctas / SMs) in.  Measured: R = 1 512^2 step 101 -> 81 us (three of four).
+template <typename T>
+constexpr int kSpreadSmem = sizeof(T) == 4 ? 116 * 1024 : 0;   // the most it asks for (FP32 kernels only)
 inline size_t spread_smem(long ctas, int num_sms, size_t smem)
 {
     const long k = (ctas + num_sms - 1) / num_sms;
@@ -227,15 +256,13 @@ gpweno_status launch_stage2d_spec(gpweno_plan p, StageArgs<T> a, const TablesFor
     auto kern = stage2d_kernel<T, R, NT, VAR, MINB, SPEC>;
     static int occ = 0;   // per instantiation: resident CTAs per SM
     if (!occ) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             std::max((int)smem, kSpreadSmem<T>));
         if (e != cudaSuccess) return cuda_fail(e, "stage2d smem attribute");
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
         if (e != cudaSuccess || occ < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
                                                           "stage2d occupancy");
         occ = std::min(occ, MINB);   // R = 1's three-CTA build needs 125 registers and would fit four times
-        if (sizeof(T) == 4)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 116 * 1024);
-        if (e != cudaSuccess) return cuda_fail(e, "stage2d smem attribute");
     }
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
     s.ctas_per_sm = occ;
@@ -270,23 +297,31 @@ gpweno_status launch_stage2d(gpweno_plan p, const StageArgs<T> &a, const TablesF
 }
 
 // The z-marching launch of a 3D stage: L = P - div_z/dz and the stage update.
-template <typename T, int R, int VAR, int SPEC>
+template <typename T, int R, int VAR, int SPEC, int NT = kNTz>
 gpweno_status launch_stagez(gpweno_plan p, const StageArgs<T> &a, const TablesFor<T, R, VAR> &tb, cudaStream_t st)
 {
-    constexpr int NT = kNTz;
     const size_t smem = stagez_smem_bytes<T, R, NT>();
     auto kern = stagez_kernel<T, R, NT, VAR, SPEC>;
     static int occ = 0;
     if (!occ) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             std::max((int)smem, kSpreadSmem<T>));
         if (e != cudaSuccess) return cuda_fail(e, "stagez smem attribute");
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
         if (e != cudaSuccess || occ < 1)
             return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "stagez occupancy");
     }
-    const long long cols = ((long long)a.n[0] * a.n[1] + NT - 1) / NT * a.n[2];
-    const int grid = (int)std::max(1LL, std::min<long long>((long long)occ * p->num_sms, cols / 8));
-    cudaError_t e = launch_pdl(kern, grid, NT, smem, st, a, tb);
+    const long long plane = (long long)a.n[0] * a.n[1];
+    const Cut3D cut = cut3d((plane + NT - 1) / NT, a.n[2], occ, p->num_sms, NT);
+    if constexpr (NT == kNTz && std::is_same<T, float>::value) {
+        // runs of half the columns where the SMs are then busy for less time (twice the CTAs resident)
+        constexpr int half = kNTz / 2;
+        if (cut3d((plane + half - 1) / half, a.n[2], 2 * occ, p->num_sms, half).cost < cut.cost)
+            return launch_stagez<T, R, VAR, SPEC, half>(p, a, tb, st);
+    }
+    const int grid = cut.grid;
+    cudaError_t e = launch_pdl(kern, grid, NT, std::is_same<T, float>::value ? spread_smem(grid, p->num_sms, smem) : smem,
+                               st, a, tb);
     if (e != cudaSuccess) return cuda_fail(e, "stagez kernel launch");
     return GPWENO_OK;
 }
@@ -368,7 +403,8 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             auto kern = plane3d_kernel<T, R, NT, VAR>;
             static int occ = 0;
             if (!occ) {
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     std::max((int)smem, kSpreadSmem<T>));
                 if (e != cudaSuccess) return cuda_fail(e, "plane3d smem attribute");
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
                 if (e != cudaSuccess || occ < 1)
@@ -381,9 +417,9 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             pa.mode = kModePartial;
             pa.out = const_cast<T *>(a.P);
             pa.rate = nullptr;
-            const long long rows = (long long)pa.nstrips * a.n[1] * a.n[2];
-            const int grid = (int)std::max(1LL, std::min<long long>((long long)occ * p->num_sms, rows / 8));
-            cudaError_t e = launch_pdl(kern, grid, NT, smem, st, pa, tb);
+            const int grid = cut3d((long long)pa.nstrips * a.n[2], a.n[1], occ, p->num_sms, NT).grid;
+            cudaError_t e = launch_pdl(
+                kern, grid, NT, std::is_same<T, float>::value ? spread_smem(grid, p->num_sms, smem) : smem, st, pa, tb);
             if (e != cudaSuccess) return cuda_fail(e, "plane3d kernel launch");
             count_launch(1);
         }

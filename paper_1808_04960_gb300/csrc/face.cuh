@@ -762,8 +762,8 @@ __device__ __forceinline__ void face_flux(const FaceRoe<T, NC> &f, const Tables 
 // smoothness forms, the Roe sound speed and the neighbour flux from differences, and doubled fluxes
 // measured per step against the form without them: FP32 1024^2 R = 2 232 -> 205 us, 4096^2
 // 2848 -> 2460 us, 3D 512^3 R = 3 63.1 -> 53.4 ms; FP64 512^2 R = 2 3086 -> 2702 us.
-// LF: local Lax-Friedrichs only (tb.flux is not read).
-template <typename T, int NC, int R, bool MEAN = false, bool AO = false, bool LF = false>
+// LF: local Lax-Friedrichs only (tb.flux is not read).  P5: five fields packed in FP32.
+template <typename T, int NC, int R, bool MEAN = false, bool AO = false, bool LF = false, bool P5 = false>
 __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
                                          T (&M)[NC], Physical<T> &ph)
 {
@@ -788,10 +788,9 @@ __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const Fac
 
     T dqL[NC], dqR[NC];
     // FP32 GP-WENO in 1D and 2D: fields in pairs (0,1), (2,3) through packed
-    // instructions, an odd last field (1D) through the scalar loop below.  3D keeps
-    // the scalar loop: with five fields the packed form spills registers in the
-    // z-marching kernel and measured 3% slower.
-    constexpr bool kPacked = std::is_same<T, float>::value && !AO && NC <= 4;
+    // instructions, an odd last field (1D, 3D) through the scalar loop below.  3D takes the packed
+    // form where its kernels have the registers for it (P5, see kPackPlane and kPackZ).
+    constexpr bool kPacked = std::is_same<T, float>::value && !AO && (NC <= 4 || P5);
     constexpr int kScalarFrom = kPacked ? (NC / 2) * 2 : 0;
     if constexpr (kPacked) {
 #pragma unroll
@@ -1030,13 +1029,13 @@ constexpr int kVarMean = 1, kVarFdFlux = 2, kVarAo = 4, kVarSlab = 8, kVarFlux =
 template <typename T, int R, int VAR>
 using TablesFor = typename std::conditional<(VAR & kVarAo) != 0, AoFaceTables<T, R>, FaceTables<T, R>>::type;
 
-template <typename T, int NC, int R, int VAR>
+template <typename T, int NC, int R, int VAR, bool P5 = false>
 __device__ __forceinline__ void face_eval(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
                                           T (&M)[NC], Physical<T> &ph)
 {
     constexpr bool kLf = std::is_same<T, float>::value && (VAR & kVarFlux) == 0;
     if constexpr ((VAR & kVarFdFlux) != 0) face_fdf<T, NC, R, (VAR & kVarMean) != 0>(st, tb, A, M, ph);
-    else face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0, kLf>(st, tb, A, M, ph);
+    else face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0, kLf, P5>(st, tb, A, M, ph);
 }
 
 // Weights of the corrected-flux difference: with the face-flux correction

@@ -235,9 +235,9 @@ __device__ __forceinline__ void rates2d(const T (&u)[4], T gam, const T (&idx)[3
 // ONE_SITE: evaluate the y- and x-face through one copy of the face routine (a
 // loop of two passes) instead of two inlined copies.  Two copies let the compiler
 // interleave the two independent faces (faster for the 2D kernels, the FP32 batch
-// included); one copy halves the code, which pays in the FP64 batch (fewer spills
-// with three radii in one kernel) and in 3D.
-template <typename T, int R, int NT, int NC = 4, int VAR = 0, bool ONE_SITE = false, int SPEC = kSpecAny>
+// included, and in 3D at R = 1 and 2); one copy halves the code, which pays in the FP64 batch (fewer spills
+// with three radii in one kernel) and in 3D at R = 3.
+template <typename T, int R, int NT, int NC = 4, int VAR = 0, bool ONE_SITE = false, int SPEC = kSpecAny, bool P5 = false>
 __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const FaceTables<T, R> &tb, int strip, int y0,
                                                 int y1, T *smem, T dt, T &rmx, T &rmy, Physical<T> &ph, long zoff = 0)
 {
@@ -392,7 +392,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                         st[q][c] = ring_at(off[q] + cc * STRIDE);
                     }
                 T An[NC], Mn[NC];
-                face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
+                face_eval<T, NC, R, VAR, P5>(st, tb, An, Mn, ph);
                 if (pass == 0) {
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
@@ -424,7 +424,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
                     }
                 }
                 T An[NC], Mn[NC];
-                face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
+                face_eval<T, NC, R, VAR, P5>(st, tb, An, Mn, ph);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     const int pc = c == 1 ? 2 : (c == 2 ? 1 : c);   // back to natural order
@@ -439,7 +439,7 @@ __device__ __forceinline__ void stage2d_segment(const StageArgs<T> &a, const Fac
 #pragma unroll
                 for (int q = 0; q < NS; ++q) ring_elem(base, tid + q, st[q]);
                 T An[NC], Mn[NC];
-                face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
+                face_eval<T, NC, R, VAR, P5>(st, tb, An, Mn, ph);
                 stage_face(FA, tid, An);
                 stage_face(FM, tid, Mn);
             }
@@ -591,6 +591,18 @@ __global__ void __launch_bounds__(NT, MINB) stage2d_kernel(StageArgs<T> a, Table
 // -div_z/dz to P and applies the stage update.  P is a buffer the update later
 // overwrites cell by cell (each cell reads its own P first), so 3D needs no
 // scratch beyond 2D's.
+//
+// Form of the 3D kernels by radius (FP32, default faces), measured on shock boxes, step us: two inlined faces per row of the
+// plane kernel and packed fields in both kernels at R = 1 (256^3 3688 -> 3476), two faces and packed fields in
+// the z kernel only at R = 2 (4671 -> 4575; 4940 with packed planes), neither at R = 3, where the
+// registers run out (6168; 6314 with two faces, 6493 packed).
+template <typename T, int R, int VAR>
+constexpr bool kOneSitePlane = sizeof(T) == 8 || R == 3 || (VAR & (kVarAo | kVarFdFlux)) != 0;
+template <typename T, int R>
+constexpr bool kPackPlane = R == 1;
+template <typename T, int R>
+constexpr bool kPackZ = R <= 2;
+
 template <typename T, int R, int NT, int VAR = 0>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT) plane3d_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
 {
@@ -610,7 +622,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT) plane3d
         const int strip = (int)(rem / ny);
         const int y0 = (int)(rem - (long)strip * ny);
         const int y1 = (int)min((long long)ny, y0 + (uend - u));
-        stage2d_segment<T, R, NT, 5, VAR, true, kSpecPartial>(a, tb, strip, y0, y1, smem, T(0), rmx, rmy, ph, (long)z * nx * ny);
+        stage2d_segment<T, R, NT, 5, VAR, kOneSitePlane<T, R, VAR>, kSpecPartial, kPackPlane<T, R>>(a, tb, strip, y0, y1, smem, T(0), rmx, rmy, ph, (long)z * nx * ny);
         u += y1 - y0;
     }
     if (__any_sync(0xffffffffu, !ph.good()) && (threadIdx.x & 31) == 0) atomicOr(a.flags, 1);
@@ -719,7 +731,7 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
                 st[q][4] = rowp[4 * NT];
             }
             T An[NC], Mn[NC];
-            face_eval<T, NC, R, VAR>(st, tb, An, Mn, ph);
+            face_eval<T, NC, R, VAR, kPackZ<T, R>>(st, tb, An, Mn, ph);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 const int pc = c == 0 || c == 4 ? c : (c == 3 ? 1 : c + 1);   // back to natural order
@@ -751,7 +763,7 @@ __device__ __forceinline__ void stagez_segment(const StageArgs<T> &a, const Face
 }
 
 template <typename T, int R, int NT, int VAR = 0, int SPEC = kSpecAny>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) stagez_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT) stagez_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *ring = reinterpret_cast<T *>(smem_raw);
