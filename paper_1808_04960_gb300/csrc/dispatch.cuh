@@ -162,7 +162,11 @@ inline Schedule schedule2d(int nx, int ny, int nt, int slots)
     return s;
 }
 
+// Block size of the tile kernel: two CTAs of 256 threads per SM; the R = 3 faces of GP-AO and FD-Flux fit 384 threads at
+// 168 registers (one CTA per SM; GP-AO step of 256^2 53 -> 42 us, of 1000 x 900 453 -> 438 against 256 threads).
 constexpr int kNTtile = 256;
+template <int R, int VAR>
+constexpr int kTileThreads = R == 3 && (VAR & (kVarAo | kVarFdFlux)) != 0 ? 384 : kNTtile;
 
 // Strip marching's CTAs of eight rows per SM (the most it makes) below which an FP32 2D grid is tiled.  Measured
 // step times, marching / tiles, at 512^2 (2.1), 768^2 (4.4), 1024^2 (7.6) and 1500^2 (16): HLLC R = 2 108/60, 143/127,
@@ -246,6 +250,9 @@ inline size_t spread_smem(long ctas, int num_sms, size_t smem)
 
 // Rows per CTA below which FP32 R = 2 grids take the three-CTA-per-SM build of the 2D kernel.
 constexpr int kWideRows = 24;
+// Rows per CTA between which R = 3 grids take it (below 16 rows they keep the four-CTA schedule that
+// gpweno_plan_schedule has reported for them, 1024^2 among them).
+constexpr int kMidRows = 16, kLongRows = 96;
 
 // One launch of the 2D stage kernel built for MINB resident CTAs per SM: occupancy (queried
 // once per instantiation), the one-wave schedule, the launch.
@@ -439,19 +446,20 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
         if constexpr (std::is_same<T, float>::value) {
             const int limit = VAR == 0 && a.mode != kModeRHS ? kTileLimitStep : kTileLimit<R, VAR>;
             if (p->tile.TX && few_rows(a.n[0], a.n[1], p->num_sms, limit)) {
-                auto kern = tile2d_kernel<R, kNTtile, VAR>;
+                constexpr int NTt = kTileThreads<R, VAR>;
+                auto kern = tile2d_kernel<R, NTt, VAR>;
                 const size_t smem = tile2d_elems<R>(p->tile.TX, p->tile.TY) * sizeof(float4);
                 cudaError_t e = cudaSuccess;
                 if (smem > 48 * 1024)
                     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 if (e != cudaSuccess) return cuda_fail(e, "tile2d smem attribute");
-                e = launch_pdl(kern, p->tile.nx * p->tile.ny, kNTtile, smem, st, a, p->tile, tb);
+                e = launch_pdl(kern, p->tile.nx * p->tile.ny, NTt, smem, st, a, p->tile, tb);
                 if (e != cudaSuccess) return cuda_fail(e, "tile2d kernel launch");
                 p->sched = Schedule();
                 p->sched.W = p->tile.TX;
                 p->sched.nstrips = p->tile.nx;
                 p->sched.grid = p->tile.nx * p->tile.ny;
-                p->sched.ctas_per_sm = kResident<T, R, VAR> / kNTtile;
+                p->sched.ctas_per_sm = NTt == kNTtile ? 2 : 1;
                 count_launch(1);
                 return GPWENO_OK;
             }
@@ -463,8 +471,8 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
         // kWideRows rows (three CTAs per SM: fewer, taller segments, fewer warm-up rows).
         // Measured on GB300 (same-box A/B, bitwise-identical results): R = 2 x1.10 at 512^2,
         // x1.05 at 768^2, x1.017 at 1024^2; R = 1 x1.14 at 700 x 640, x1.05 at 777 x 613; R = 3 x1.10 at
-        // 777 x 613, x1.05 at 1024 x 512.  Not taken where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98),
-        // R = 1 at 1024^2 (x0.98), R = 3 at 1024^2 (x0.986).
+        // 777 x 613, x1.05 at 1024 x 512, x1.03 at 1501 x 1100, x1.016 at 2048^2 (HLLC x1.013, x1.005).  Not
+        // taken where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98), R = 1 at 1024^2 (x0.98).
         constexpr bool kHasWide = std::is_same<T, float>::value && (VAR & ~(kVarSlab | kVarFlux)) == 0;
         if constexpr (kHasWide) {
             const int slots4 = 512 / NT * p->num_sms;
@@ -472,7 +480,9 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             const long long rows = (long long)s4.nstrips * a.n[1];
             const bool row_limited = s4.grid < slots4;
             const bool short_segments = R == 2 && rows < (long long)kWideRows * s4.grid;
-            if (row_limited || short_segments) {
+            const bool mid_segments =
+                R == 3 && rows >= (long long)kMidRows * s4.grid && rows < (long long)kLongRows * s4.grid;
+            if (row_limited || short_segments || mid_segments) {
                 gpweno_status r = launch_stage2d<T, R, NT, VAR, 3>(p, a, tb, st);
                 if (r != GPWENO_OK) return r;
                 count_launch(1);

@@ -24,7 +24,7 @@ constexpr __host__ __device__ size_t tile2d_elems(int TX, int TY)
 }
 
 template <int R, int NT, int VAR>
-__global__ void __launch_bounds__(NT, kResident<float, R, VAR> / NT)
+__global__ void __launch_bounds__(NT, NT == 384 ? 1 : kResident<float, R, VAR> / NT)
     tile2d_kernel(StageArgs<float> a, Tile2D t, TablesFor<float, R, VAR> tb)
 {
     constexpr int G = R + 3, NS = 2 * R + 2, NC = 4;
