@@ -29,9 +29,9 @@
  *     Launches are asynchronous; errors of earlier launches surface at the
  *     next call or at gpweno_flags().  Step functions allocate nothing and do
  *     not synchronise.
- *   - A plan owns its weight tables and a small device workspace (flags,
- *     wavespeed maxima); it is not thread-safe to use one plan from two
- *     streams at once.
+ *   - A plan owns its weight tables and a device workspace (flags, wavespeed
+ *     maxima, FP64 face fluxes); it is not thread-safe to use one plan from
+ *     two streams at once.
  */
 #ifndef GPWENO_H
 #define GPWENO_H
