@@ -500,10 +500,11 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             a.nseg = 1;
             e = launch_pdl(kern, a.nstrips, nt, smem, st, a, tb);
         };
-        // FP64: field-split CTAs up to two per SM (8 K cells).  Six of their warps load an SM's FP64 pipe by
-        // 25 thousand cycles, four of the plain kernel's by 38 thousand; three CTAs would draw level
+        // FP64: field-split CTAs up to three per SM (12 K cells).  Measured steps, split and plain, R = 1, 2, 3:
+        // 8208 cells (two per SM) 35.7, 42.9, 52.5 and 53.4, 66.4, 84.8 us; 12312 cells (three) 48.3, 59.5, 74.2
+        // and 53.0, 65.9, 84.6 us; a fourth would draw level
         constexpr bool kSplit = std::is_same<T, double>::value && (VAR & (kVarAo | kVarFdFlux)) == 0;
-        if (kSplit && (a.n[0] + 26) / 27 <= 2 * p->num_sms) {
+        if (kSplit && (a.n[0] + 26) / 27 <= 3 * p->num_sms) {
             if constexpr (kSplit) launch(stage1d_split_kernel<T, R, VAR>, 27, 96, 0);
         } else {
             launch(stage1d_kernel<T, R, kNT1D, VAR>, kNT1D - 5, kNT1D, stage1d_smem_bytes<T, R, kNT1D>());

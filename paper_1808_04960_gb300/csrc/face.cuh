@@ -370,36 +370,46 @@ struct FaceRoe {
     }
 };
 
-template <typename T, int NC, typename Tables>
-__device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&uR)[NC], const Tables &tb)
+// What the Roe average takes from each cell alone, for kernels that form it once per cell and not per face.
+template <typename T, int NC>
+struct CellPart {
+    T rs, ir, s;                   // rho^-1/2, 1/rho, rho^1/2
+    T u[NC - 2], p, hp, c2;        // used of cell s only
+};
+
+// PARTS: the cells' parts are given, otherwise formed here (in this order, which the compiler's register
+// allocation in the 3D kernels answers to: 2 % at 512^3).
+template <typename T, int NC, bool PARTS = false, typename Tables>
+__device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&uR)[NC], const Tables &tb,
+                                                   const CellPart<T, NC> &L = {}, const CellPart<T, NC> &R = {})
 {
     constexpr int NV = NC - 2, E = NC - 1;
     FaceRoe<T, NC> f;
     f.gm1 = tb.gm1;
     const T rL = uL[0], rR = uR[0];
-    const T rsL = Num<T>::rsqrt(rL), rsR = Num<T>::rsqrt(rR);
-    const T irL = rsL * rsL, irR = rsR * rsR;
+    const T rsL = PARTS ? L.rs : Num<T>::rsqrt(rL), rsR = PARTS ? R.rs : Num<T>::rsqrt(rR);
+    const T irL = PARTS ? L.ir : rsL * rsL, irR = PARTS ? R.ir : rsR * rsR;
     f.ref.rho = rL;
     T mu = T(0);
 #pragma unroll
     for (int a = 0; a < NV; ++a) {
-        f.ref.u[a] = uL[1 + a] * irL;
+        f.ref.u[a] = PARTS ? L.u[a] : vmul_keep(uL[1 + a], irL);
         mu = fma(uL[1 + a], f.ref.u[a], mu);
     }
-    f.ref.p = f.gm1 * fma(T(-0.5), mu, uL[E]);
-    f.ref.hp = uL[E] + f.ref.p;
+    f.ref.p = PARTS ? L.p : vmul_keep(f.gm1, fma(T(-0.5), mu, uL[E]));
+    f.ref.hp = PARTS ? L.hp : uL[E] + f.ref.p;
     f.ref.mn = uL[1];
     f.Vs[0] = rL;
 #pragma unroll
     for (int a = 0; a < NV; ++a) f.Vs[1 + a] = f.ref.u[a];
     f.Vs[E] = f.ref.p;
     f.prim_diff(uR, uL, irR, f.dVn);
-    const T sL = rL * rsL, sR = rR * rsR;   // sqrt(rho)
+    const T sL = PARTS ? L.s : vmul_keep(rL, rsL), sR = PARTS ? R.s : vmul_keep(rR, rsR);   // sqrt(rho)
     f.th = sR * Num<T>::rcp(sL + sR);
     T du2 = T(0);
 #pragma unroll
     for (int a = 0; a < NV; ++a) du2 = fma(f.dVn[1 + a], f.dVn[1 + a], du2);
-    const T cL2 = tb.gamma * irL * f.ref.p, cR2 = tb.gamma * irR * (f.ref.p + f.dVn[E]);
+    const T cL2 = PARTS ? L.c2 : vmul_keep(tb.gamma * irL, f.ref.p), cR2 = tb.gamma * irR * (f.ref.p + f.dVn[E]);
     f.c2 = fma(tb.hgm1 * fma(-f.th, f.th, f.th), du2, fma(f.th, cR2 - cL2, cL2));
     f.ic = Num<T>::rsqrt(Num<T>::pmax(f.c2, T(1e-30)));
     f.c = f.c2 * f.ic;
@@ -410,6 +420,27 @@ __device__ __forceinline__ FaceRoe<T, NC> face_roe(const T (&uL)[NC], const T (&
     f.ap = T(0.5) * f.ie;
     f.cr = f.c * f.irb;
     return f;
+}
+
+// The part of cell U, with face_roe's roundings
+template <typename T, int NC, typename Tables>
+__device__ __forceinline__ CellPart<T, NC> cell_part(const T (&U)[NC], const Tables &tb)
+{
+    constexpr int NV = NC - 2, E = NC - 1;
+    CellPart<T, NC> c;
+    c.rs = Num<T>::rsqrt(U[0]);
+    c.ir = c.rs * c.rs;
+    c.s = vmul_keep(U[0], c.rs);
+    T mu = T(0);
+#pragma unroll
+    for (int a = 0; a < NV; ++a) {
+        c.u[a] = vmul_keep(U[1 + a], c.ir);
+        mu = fma(U[1 + a], c.u[a], mu);
+    }
+    c.p = vmul_keep(tb.gm1, fma(T(-0.5), mu, U[E]));
+    c.hp = U[E] + c.p;
+    c.c2 = vmul_keep(tb.gamma * c.ir, c.p);
+    return c;
 }
 
 // (eps + beta)^-p of one smoothness window: beta = f^T K_m(sigma)^-1 f (Eq. beta-eigen, in another

@@ -873,18 +873,21 @@ __global__ void __launch_bounds__(NT) stage1d_kernel(StageArgs<T> a, TablesFor<T
 }
 
 // The same for short FP64 grids: a CTA of three warps owns W <= 27 cells and its W+5 <= 32 faces, warp k
-// evaluating characteristic field k of every face (the Roe average and the primitive differences by all
-// three), then the left state, the right state and the neighbour flux, then component k of the
-// flux.  A warp passes one dependent FP64 instruction in about 58 cycles, whatever its SM's load, so a grid
-// of a few warps is as slow as one face's instructions in a row: 17 us per stage of 256 cells at R = 2.
-// The split takes two thirds of a face's instructions out of each warp's row.
-// Measured: 256-cell step R = 2 60.0 -> 36.8 us.
+// evaluating characteristic field k of every face (the Roe average by all three, each cell's own part of
+// it once, the primitive differences in turns), then the left state, the right state and the neighbour flux, then
+// component k of the flux.  A warp passes one FP64 instruction per 64 cycles, independent or not and however
+// many of its lanes are active, and an SM one per 19 (measured with chains of fma), so a grid of a few
+// warps is as slow as one face's instructions in a row: 17 us per stage of 256 cells at R = 2.  Three warps
+// on one SM lose nothing to each other and split that row.
+// Measured: 256-cell step R = 2 60.0 -> 36.7 us by fields, 33.3 us with the shared parts.
 template <typename T, int R, int VAR>
 __global__ void __launch_bounds__(96) stage1d_split_kernel(StageArgs<T> a, TablesFor<T, R, VAR> tb)
 {
     constexpr int G = R + 3, NC = 3, NS = 2 * R + 2, NF = 32, E = 2;
     constexpr bool MEAN = (VAR & kVarMean) != 0;
     __shared__ T row[NC][NF + NS];        // staged cells x0-G .. x0+W+G-1
+    __shared__ T part0[8][NF + NS];       // of each cell: 1/rho and CellPart
+    __shared__ T dVs[2 * R][NC][NF];      // primitive differences of the cells beyond the neighbours
     __shared__ T q[2][NC][NF];            // left and right states in characteristic fields
     __shared__ T part[2][3 * NC + 2][NF]; // left, right: w, G, c, u, a
     __shared__ T nb[NC][NF];              // neighbour flux difference
@@ -901,27 +904,51 @@ __global__ void __launch_bounds__(96) stage1d_split_kernel(StageArgs<T> a, Table
             row[k][col] = src[k * cs];
     }
     __syncthreads();
+    if (const int col = threadIdx.x; col < Wc + 2 * G && chk(col, NF + NS, kChkLine, a.flags)) {
+        const T U[NC] = {row[0][col], row[1][col], row[2][col]};
+        const CellPart<T, NC> cp = cell_part(U, tb);
+        const T v[8] = {Num<T>::rcp(U[0]), cp.rs, cp.ir, cp.s, cp.u[0], cp.p, cp.hp, cp.c2};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) part0[c][col] = v[c];
+    }
+    __syncthreads();
     const bool face = lane < Wc + 5 && chk(lane + NS - 1, NF + NS, kChkLine, a.flags);
     Physical<T> ph;
     FaceRoe<T, NC> f;
+    if (face) {
+        const int s = lane + R;
+        const T uL[NC] = {row[0][s], row[1][s], row[2][s]}, uR[NC] = {row[0][s + 1], row[1][s + 1], row[2][s + 1]};
+        CellPart<T, NC> L = {}, Rt = {};
+        L.rs = part0[1][s];
+        L.ir = part0[2][s];
+        L.s = part0[3][s];
+        L.u[0] = part0[4][s];
+        L.p = part0[5][s];
+        L.hp = part0[6][s];
+        L.c2 = part0[7][s];
+        Rt.rs = part0[1][s + 1];
+        Rt.ir = part0[2][s + 1];
+        Rt.s = part0[3][s + 1];
+        f = face_roe<T, NC, true>(uL, uR, tb, L, Rt);
+        // warp k takes every third of the other cells
+        for (int i = k; i < 2 * R; i += NC) {
+            const int j = lane + (i < R ? i : i + 2);
+            const T uj[NC] = {row[0][j], row[1][j], row[2][j]};
+            T dV[NC];
+            f.prim_diff(uj, uL, part0[0][j], dV);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) dVs[i][c][lane] = dV[c];
+        }
+    }
+    __syncthreads();
     T us[NC], ur[NC];
     if (face) {
-        T st[NS][NC];
+        T dV[NS][NC], d[NS];
 #pragma unroll
         for (int j = 0; j < NS; ++j)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) st[j][c] = row[c][lane + j];
-        f = face_roe<T, NC>(st[R], st[R + 1], tb);
-        T dV[NS][NC], d[NS];
-#pragma unroll
-        for (int j = 0; j < NS; ++j) {
-            if (j == R || j == R + 1) {
-#pragma unroll
-                for (int c = 0; c < NC; ++c) dV[j][c] = j == R ? T(0) : f.dVn[c];
-                continue;
-            }
-            f.prim_diff(st[j], st[R], dV[j]);
-        }
+            for (int c = 0; c < NC; ++c)
+                dV[j][c] = j == R ? T(0) : (j == R + 1 ? f.dVn[c] : dVs[j < R ? j : j - 2][c][lane]);
         // the rows of L_V: (0, -an, ap), (1, 0, -ie), (0, an, ap)
 #pragma unroll
         for (int j = 0; j < NS; ++j)
@@ -933,8 +960,8 @@ __global__ void __launch_bounds__(96) stage1d_split_kernel(StageArgs<T> a, Table
         q[1][k][lane] = qR;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            us[c] = st[R][c];
-            ur[c] = st[R + 1][c];
+            us[c] = row[c][lane + R];
+            ur[c] = row[c][lane + R + 1];
         }
     }
     __syncthreads();
@@ -961,19 +988,26 @@ __global__ void __launch_bounds__(96) stage1d_split_kernel(StageArgs<T> a, Table
     }
     __syncthreads();
     if (face) {
-        T w[2][NC], Gf[2][NC], cw[2][NC], A[NC];
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                w[s][c] = part[s][c][lane];
-                Gf[s][c] = part[s][NC + c][lane];
-                cw[s][c] = part[s][2 * NC + c][lane];
-            }
         const T uL = part[0][3 * NC][lane], aL = part[0][3 * NC + 1][lane];
         const T uR = part[1][3 * NC][lane], aR = part[1][3 * NC + 1][lane];
-        face_flux<T, NC, false>(f, tb, w[0], w[1], Gf[0], Gf[1], cw[0], cw[1], uL, uR, aL, aR, A);
-        const T Ak = k == 0 ? A[0] : (k == 1 ? A[1] : A[2]);
+        T Ak;
+        if (tb.flux == 0) {   // Lax-Friedrichs, component k alone (as face_flux)
+            const T alpha = Num<T>::pmax(Num<T>::fabs(uL) + aL, Num<T>::fabs(uR) + aR);
+            Ak = fma(-alpha, part[1][2 * NC + k][lane] - part[0][2 * NC + k][lane],
+                     part[0][NC + k][lane] + part[1][NC + k][lane]);
+        } else {
+            T w[2][NC], Gf[2][NC], cw[2][NC], A[NC];
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    w[s][c] = part[s][c][lane];
+                    Gf[s][c] = part[s][NC + c][lane];
+                    cw[s][c] = part[s][2 * NC + c][lane];
+                }
+            face_flux<T, NC, false>(f, tb, w[0], w[1], Gf[0], Gf[1], cw[0], cw[1], uL, uR, aL, aR, A);
+            Ak = k == 0 ? A[0] : (k == 1 ? A[1] : A[2]);
+        }
         FA[k][lane] = Ak;
         FM[k][lane] = fma(T(-2), nb[k][lane], Ak);
     }
