@@ -2,6 +2,7 @@
 // conversion, schedule (strip width, segment height, grid), kernel selection.
 #pragma once
 #include <algorithm>
+#include <atomic>
 
 #include "list.cuh"
 #include "plan.h"
@@ -248,6 +249,35 @@ inline size_t spread_smem(long ctas, int num_sms, size_t smem)
     return std::max(smem, want);
 }
 
+constexpr int kAnyResident = 1 << 20;   // no cap
+// Resident CTAs per SM of one kernel, by device: its limit on dynamic shared memory belongs to a device as well and is
+// raised there before the first launch.  Any number of threads may ask at once: each finds the same value,
+// and only the final one (capped at `most`) is ever stored.
+class Residency {
+public:
+    template <typename K>
+    gpweno_status get(const gpweno_plan_s *p, K kern, int block, size_t smem, size_t smem_limit, int most, const char *what,
+                      int &ctas)
+    {
+        const bool cached = p->device >= 0 && p->device < kDevices;
+        ctas = cached ? of_[p->device].load(std::memory_order_acquire) : 0;
+        if (ctas) return GPWENO_OK;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)std::max(smem, smem_limit));
+        if (e != cudaSuccess) return cuda_fail(e, what);
+        int n = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem);
+        if (e != cudaSuccess || n < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, what);
+        ctas = std::min(n, most);
+        if (cached) of_[p->device].store(ctas, std::memory_order_release);
+        return GPWENO_OK;
+    }
+
+private:
+    static constexpr int kDevices = 64;   // beyond it every launch asks
+    std::atomic<int> of_[kDevices] = {};
+};
+
 // Rows per CTA below which FP32 R = 2 grids take the three-CTA-per-SM build of the 2D kernel.
 constexpr int kWideRows = 24;
 // Rows per CTA between which R = 3 grids take it (below 16 rows they keep the four-CTA schedule that
@@ -261,16 +291,11 @@ gpweno_status launch_stage2d_spec(gpweno_plan p, StageArgs<T> a, const TablesFor
 {
     const size_t smem = stage2d_smem_bytes<T, R, NT>();
     auto kern = stage2d_kernel<T, R, NT, VAR, MINB, SPEC>;
-    static int occ = 0;   // per instantiation: resident CTAs per SM
-    if (!occ) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             std::max((int)smem, kSpreadSmem<T>));
-        if (e != cudaSuccess) return cuda_fail(e, "stage2d smem attribute");
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
-        if (e != cudaSuccess || occ < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
-                                                          "stage2d occupancy");
-        occ = std::min(occ, MINB);   // R = 1's three-CTA build needs 125 registers and would fit four times
-    }
+    static Residency residency;   // per instantiation
+    int occ;
+    // at most MINB: R = 1's three-CTA build needs 125 registers and would fit four times
+    const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, MINB, "stage2d occupancy", occ);
+    if (r != GPWENO_OK) return r;
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
     s.ctas_per_sm = occ;
     a.W = s.W;
@@ -309,15 +334,10 @@ gpweno_status launch_stagez(gpweno_plan p, const StageArgs<T> &a, const TablesFo
 {
     const size_t smem = stagez_smem_bytes<T, R, NT>();
     auto kern = stagez_kernel<T, R, NT, VAR, SPEC>;
-    static int occ = 0;
-    if (!occ) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             std::max((int)smem, kSpreadSmem<T>));
-        if (e != cudaSuccess) return cuda_fail(e, "stagez smem attribute");
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
-        if (e != cudaSuccess || occ < 1)
-            return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "stagez occupancy");
-    }
+    static Residency residency;
+    int occ;
+    const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, kAnyResident, "stagez occupancy", occ);
+    if (r != GPWENO_OK) return r;
     const long long plane = (long long)a.n[0] * a.n[1];
     const Cut3D cut = cut3d((plane + NT - 1) / NT, a.n[2], occ, p->num_sms, NT);
     if constexpr (NT == kNTz && std::is_same<T, float>::value) {
@@ -408,15 +428,10 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             constexpr int NT = kNTxy<T>;
             const size_t smem = stage2d_smem_bytes<T, R, NT, 5>();
             auto kern = plane3d_kernel<T, R, NT, VAR>;
-            static int occ = 0;
-            if (!occ) {
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     std::max((int)smem, kSpreadSmem<T>));
-                if (e != cudaSuccess) return cuda_fail(e, "plane3d smem attribute");
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem);
-                if (e != cudaSuccess || occ < 1)
-                    return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "plane3d occupancy");
-            }
+            static Residency residency;
+            int occ;
+            const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, kAnyResident, "plane3d occupancy", occ);
+            if (r != GPWENO_OK) return r;
             StageArgs<T> pa = a;
             const int wmax = NT - 5;
             pa.nstrips = (a.n[0] + wmax - 1) / wmax;
