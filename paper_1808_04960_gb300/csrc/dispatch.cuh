@@ -166,6 +166,7 @@ inline Schedule schedule2d(int nx, int ny, int nt, int slots)
 // Block size of the tile kernel: two CTAs of 256 threads per SM; the R = 3 faces of GP-AO and FD-Flux fit 384 threads at
 // 168 registers (one CTA per SM; GP-AO step of 256^2 53 -> 42 us, of 1000 x 900 453 -> 438 against 256 threads).
 constexpr int kNTtile = 256;
+constexpr int kTileSmem = 100 * 1024;   // most shared memory of a tile
 template <int R, int VAR>
 constexpr int kTileThreads = R == 3 && (VAR & (kVarAo | kVarFdFlux)) != 0 ? 384 : kNTtile;
 
@@ -196,7 +197,7 @@ inline Tile2D choose_tile(int nx, int ny, int R, int num_sms)
         for (int TY = 4; TY <= 64; ++TY) {
             const long G = R + 3;
             const long elems = (TX + 2 * G) * (TY + 2 * G) + 2 * ((TX + 5L) * TY + TX * (TY + 5L));
-            if (elems * 16 > 100 * 1024) break;   // two CTAs per SM
+            if (elems * 16 > kTileSmem) break;   // two CTAs per SM
             const int tx = (nx + TX - 1) / TX, ty = (ny + TY - 1) / TY;
             const long tiles = (long)tx * ty, per_sm = (tiles + num_sms - 1) / num_sms;
             const long warps = ((TX + 5L) * TY + TX * (TY + 5L) + 31) / 32;
@@ -464,11 +465,11 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
                 constexpr int NTt = kTileThreads<R, VAR>;
                 auto kern = tile2d_kernel<R, NTt, VAR>;
                 const size_t smem = tile2d_elems<R>(p->tile.TX, p->tile.TY) * sizeof(float4);
-                cudaError_t e = cudaSuccess;
-                if (smem > 48 * 1024)
-                    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return cuda_fail(e, "tile2d smem attribute");
-                e = launch_pdl(kern, p->tile.nx * p->tile.ny, NTt, smem, st, a, p->tile, tb);
+                static Residency residency;   // at the largest tile; never lowered for a plan of smaller ones
+                int occ;
+                const gpweno_status r = residency.get(p, kern, NTt, kTileSmem, kTileSmem, kAnyResident, "tile2d occupancy", occ);
+                if (r != GPWENO_OK) return r;
+                cudaError_t e = launch_pdl(kern, p->tile.nx * p->tile.ny, NTt, smem, st, a, p->tile, tb);
                 if (e != cudaSuccess) return cuda_fail(e, "tile2d kernel launch");
                 p->sched = Schedule();
                 p->sched.W = p->tile.TX;

@@ -102,3 +102,15 @@ fake.fake_release()
 t.join()
 assert got == 3 == schedule(a)[3], (got, schedule(a))
 """)
+
+
+def test_tiles_of_different_sizes(run):
+    """No launch lowers a kernel's limit on dynamic shared memory: two threads that step plans of large and small
+    tiles of the same kernel may interleave anywhere."""
+    run("""
+plans = [plan((n, n)) for n in (480, 384, 256, 300)]
+for p in plans + plans:
+    step(p)
+    rhs(p)
+assert fake.fake_lowered() == 0, fake.fake_lowered()
+""")
