@@ -187,7 +187,8 @@ inline bool few_rows(int nx, int ny, int num_sms, int per_sm)
 
 // Tiles of a small FP32 2D grid, or none (TX = 0).  The tile minimises the busiest SM's
 // work and depth: it evaluates `work` warps of faces, at 230 cycles each when
-// its issue slots are full, and a CTA's list is `depth` faces deep, at 1500 cycles each.
+// its issue slots are full, and a CTA's list is `depth` faces deep, at 1500 cycles each.  The estimate takes two CTAs
+// of 256 threads per SM; FD-Flux R = 2 (130 registers) has one, as have the 384-thread builds.
 inline Tile2D choose_tile(int nx, int ny, int R, int num_sms)
 {
     Tile2D best;
@@ -475,7 +476,7 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
                 p->sched.W = p->tile.TX;
                 p->sched.nstrips = p->tile.nx;
                 p->sched.grid = p->tile.nx * p->tile.ny;
-                p->sched.ctas_per_sm = NTt == kNTtile ? 2 : 1;
+                p->sched.ctas_per_sm = occ;
                 count_launch(1);
                 return GPWENO_OK;
             }

@@ -22,7 +22,7 @@ std::map<std::pair<int, const void *>, int> g_limit;
 std::map<const void *, std::pair<size_t, int>> g_blocks;   // allocation -> bytes, device
 size_t g_bytes = 0, g_budget = ~size_t(0);
 long g_launches = 0, g_lowered = 0;
-std::atomic<int> g_hold{0}, g_held{0};
+std::atomic<int> g_hold{0}, g_held{0}, g_resident{0};
 struct Config {
     dim3 grid, block;
     size_t smem;
@@ -52,6 +52,7 @@ void fake_budget(size_t bytes) { g_budget = bytes; } // cudaMalloc fails beyond 
 void fake_hold() { g_hold = 1; }                     // the next residency query returns only after fake_release()
 int fake_held() { return g_held; }
 void fake_release() { g_held = 0; }
+void fake_resident(int n) { g_resident = n; }        // residency queries answer n
 
 // ---- the runtime ----
 const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "fake runtime error"; }
@@ -128,7 +129,7 @@ cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int v)
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int block, size_t smem,
                                                                    unsigned)
 {
-    *n = std::max(1, std::min(512 / block, (int)(228 * 1024 / (smem + 1024))));
+    *n = g_resident ? g_resident.load() : std::max(1, std::min(512 / block, (int)(228 * 1024 / (smem + 1024))));
     if (g_hold.exchange(0)) {
         g_held = 1;
         for (int k = 0; k < 5000 && g_held; ++k) std::this_thread::sleep_for(std::chrono::milliseconds(1));

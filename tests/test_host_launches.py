@@ -114,3 +114,16 @@ for p in plans + plans:
     rhs(p)
 assert fake.fake_lowered() == 0, fake.fake_lowered()
 """)
+
+
+@pytest.mark.parametrize("shape,R,opts,ctas", [((100, 100), 2, {}, 1), ((100, 100), 2, dict(scheme=1), 1),
+                                               ((100, 100), 2, dict(ao=1), 1), ((100, 100), 2, dict(ao=1), 2),
+                                               ((100, 100), 3, dict(ao=1), 1), ((100, 100), 1, dict(scheme=1), 2)])
+def test_schedule_reports_the_tiles_residency(run, shape, R, opts, ctas):
+    """The CTAs per SM that gpweno_plan_schedule gives for a tile launch are the runtime's."""
+    run(f"""
+fake.fake_resident({ctas})
+p = plan({shape}, {R}, **{opts})
+step(p)
+assert schedule(p)[3] == {ctas}, schedule(p)
+""")
