@@ -146,7 +146,8 @@ void gpweno_default_opts(gpweno_opts *opts);
  * hundred bytes of device memory on the current device, and for FP64 2D and 3D
  * plans a workspace for the face fluxes of a band of the grid (at most 32 MiB, or
  * 24 layers of the slowest dimension where that is more; none above 1 GiB or
- * if the allocation fails, the steps then run on slower kernels); the plan must be
+ * if the allocation fails, the steps then run on slower kernels with the same results; see
+ * gpweno_plan_workspace); the plan must be
  * used on that device.  Returns GPWENO_ERR_PRECOMPUTE if the covariance
  * system is too ill-conditioned for double-double. */
 gpweno_status gpweno_plan_create(gpweno_plan *out, int R, double ell_over_dx, const gpweno_dims *dims,
@@ -315,7 +316,9 @@ gpweno_status gpweno_flags(gpweno_plan plan, int *nonphysical);
  * fields "<strip width cap (0 = as the block allows)> <fewest rows of a segment
  * that does not end its strip> <CTA shares per resident slot (1..16)>" (the
  * tile shapes the autotuner searches).  Allocates its schedule and descriptor
- * arrays on the device. */
+ * arrays on the device.  Batches need no FP64 face workspace: members that have not stepped
+ * alone (gpweno_rhs, gpweno_rk3_step or gpweno_rk3_stage) give theirs back, and step with the
+ * slower kernels if they do so later. */
 gpweno_status gpweno_plan_batch(gpweno_plan *out_batch, const gpweno_plan *plans, int n, const char *tune_cache);
 
 /* One SSP-RK3 step of every instance of a batch plan, in place:
@@ -342,6 +345,11 @@ int gpweno_batch_info(gpweno_plan batch, int *block, int *ctas_per_sm, int *grid
  * residency of the face launch.  All zero before the first launch.  Returns
  * GPWENO_ERR_ARG for batch plans and 1D or 3D plans. */
 int gpweno_plan_schedule(gpweno_plan plan, int *strip_width, int *strips, int *grid, int *ctas_per_sm);
+
+/* Device memory of the face workspace that an FP64 2D or 3D plan holds (see gpweno_plan_create and
+ * gpweno_plan_batch); 0 where it has none, its steps then run on the slower kernels, and for
+ * other plans. */
+gpweno_status gpweno_plan_workspace(gpweno_plan plan, unsigned long long *bytes);
 
 /* Tile shapes of a batch plan's schedule: the widest strip (columns), the
  * fewest rows of a segment that does not finish its strip, and CTA shares per

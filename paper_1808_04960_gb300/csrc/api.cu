@@ -231,7 +231,7 @@ gpweno_status gpweno_plan_destroy(gpweno_plan p)
 {
     if (!p) return GPWENO_OK;
     if (p->ws) cudaFree(p->ws);
-    if (p->face_ws) cudaFree(p->face_ws);
+    if (p->has_face_ws()) cudaFree(p->face_ws);
     if (p->batch_inst_dev) cudaFree(p->batch_inst_dev);
     if (p->batch_inst_host) cudaFreeHost(p->batch_inst_host);
     if (p->batch_segs_dev) cudaFree(p->batch_segs_dev);
@@ -686,6 +686,7 @@ gpweno_status gpweno_plan_batch(gpweno_plan *out, const gpweno_plan *plans, int 
         gpweno_plan_destroy(b);
         return s;
     }
+    for (gpweno_plan p : b->members) p->give_face_ws_back();
     *out = b;
     return GPWENO_OK;
 }
@@ -723,6 +724,16 @@ int gpweno_plan_schedule(gpweno_plan p, int *strip_width, int *strips, int *grid
     if (strips) *strips = p->sched.nstrips;
     if (grid) *grid = p->sched.grid;
     if (ctas_per_sm) *ctas_per_sm = p->sched.ctas_per_sm;
+    return GPWENO_OK;
+}
+
+gpweno_status gpweno_plan_workspace(gpweno_plan p, unsigned long long *bytes)
+{
+    if (!p || !bytes) {
+        set_error("gpweno_plan_workspace: invalid argument");
+        return GPWENO_ERR_ARG;
+    }
+    *bytes = p->has_face_ws() ? p->face_ws_bytes : 0;
     return GPWENO_OK;
 }
 

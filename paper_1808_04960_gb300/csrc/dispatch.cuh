@@ -552,7 +552,7 @@ gpweno_status launch_stage_T(gpweno_plan p, const StageIO &io, cudaStream_t st)
     a.dt = io.dt;
     a.dt_dev = io.dt_dev;
     a.rate = io.want_rate ? p->ws : nullptr;
-    const bool use_list = p->face_ws != nullptr && !io.no_workspace;
+    const bool use_list = !io.no_workspace && p->claim_face_ws();
     switch (p->R) {
     case 1:
         if constexpr ((VAR & kVarAo) != 0) {

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -42,6 +43,22 @@ struct gpweno_plan_s {
     void *face_ws = nullptr;
     size_t face_ws_bytes = 0;
     int face_ws_layers = 0;                 // layers of the slowest dimension per band
+    // The first launch that uses the workspace keeps it for the plan's lifetime (a captured graph may hold its
+    // address); a batch built before that gives it back.
+    enum FaceUse { kFaceIdle, kFaceUsed, kFaceGiven };
+    std::atomic<int> face_use{kFaceIdle};
+    bool claim_face_ws()
+    {
+        int s = face_use.load(std::memory_order_acquire);
+        if (s == kFaceIdle && face_use.compare_exchange_strong(s, kFaceUsed)) s = kFaceUsed;
+        return s == kFaceUsed && face_ws != nullptr;
+    }
+    void give_face_ws_back()
+    {
+        int s = kFaceIdle;
+        if (face_use.compare_exchange_strong(s, kFaceGiven) && face_ws) cudaFree(face_ws);
+    }
+    bool has_face_ws() const { return face_use.load(std::memory_order_acquire) != kFaceGiven && face_ws != nullptr; }
     const void *halo[2] = {nullptr, nullptr};   // halo buffers of external sides (gpweno_set_halo)
     bool is_batch = false;
     // batch-only data

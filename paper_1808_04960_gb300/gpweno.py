@@ -82,6 +82,7 @@ def load(path: str | None = None):
             "gpweno_batch_tiles": (i, [vp, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i)]),
             "gpweno_plan_schedule": (i, [vp, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i),
                                          ctypes.POINTER(i)]),
+            "gpweno_plan_workspace": (i, [vp, ctypes.POINTER(ctypes.c_ulonglong)]),
             "gpweno_last_error": (ctypes.c_char_p, []),
         }
         for name, (res, args) in sigs.items():
@@ -386,6 +387,12 @@ class Plan:
         v = [ctypes.c_int() for _ in range(4)]
         _check(self.lib.gpweno_plan_schedule(self.handle, *[ctypes.byref(x) for x in v]), "gpweno_plan_schedule")
         return dict(strip_width=v[0].value, strips=v[1].value, grid=v[2].value, ctas_per_sm=v[3].value)
+
+    def workspace(self) -> int:
+        """Bytes of device memory of the FP64 face workspace (0: none, the steps run on the slower kernels)."""
+        v = ctypes.c_ulonglong(0)
+        _check(self.lib.gpweno_plan_workspace(self.handle, ctypes.byref(v)), "gpweno_plan_workspace")
+        return int(v.value)
 
     def flags(self) -> int:
         v = ctypes.c_int(0)

@@ -127,3 +127,36 @@ p = plan({shape}, {R}, **{opts})
 step(p)
 assert schedule(p)[3] == {ctas}, schedule(p)
 """)
+
+
+def test_batch_members_give_their_workspace_back(run):
+    """The batch kernel reads no face workspace: members that have never stepped alone hold none once the batch is
+    built (they step with the marching kernels from then on); a member that has, keeps its own, which a
+    captured graph may refer to.  Lost workspaces show in gpweno_plan_workspace."""
+    run("""
+def held(p):
+    v = ctypes.c_ulonglong()
+    g._check(lib.gpweno_plan_workspace(p, ctypes.byref(v)))
+    return v.value
+
+start = fake.fake_bytes()
+members = [plan((256, 256 + k), 1 + k % 3, "f64") for k in range(8)]
+step(members[0])
+assert all(held(p) >= 8 << 20 for p in members)
+arr = (ctypes.c_void_p * 8)(*[p.value for p in members])
+b = ctypes.c_void_p()
+g._check(lib.gpweno_plan_batch(ctypes.byref(b), arr, 8, None))
+assert fake.fake_bytes() - start < held(members[0]) + (1 << 20), fake.fake_bytes() - start
+assert held(members[0]) >= 8 << 20 and not any(held(p) for p in members[1:])
+for p, launches in ((members[0], 6), (members[1], 3)):   # face lists and updates, marching
+    step(p)
+    assert lib.gpweno_last_launch_count() == launches
+lib.gpweno_plan_destroy(b)
+for p in members:
+    lib.gpweno_plan_destroy(p)
+assert fake.fake_bytes() == start
+
+fake.fake_budget(fake.fake_bytes() + (1 << 20))
+p = plan((256, 256), 2, "f64")
+assert held(p) == 0
+""")
