@@ -26,7 +26,7 @@ OUT_DIR_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(HERE, "libgpweno_checked.so")
 SOURCES = ["api.cu", "stage_f32.cu", "stage_f64.cu", "gp_precompute.cpp", "noalloc.cu", "batch_f32.cu",
            "batch_f64.cu"] + ["stage_%s_var%d.cu" % (t, v) for t in ("f32", "f64") for v in (1, 2, 3, 4, 5, 8)] + [
-               "stage_f32_var%d.cu" % v for v in (16, 17, 20, 21, 24)]
+               "stage_f32_var%d.cu" % v for v in (16, 17, 20, 21, 24, 34, 48, 56)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -38,6 +38,7 @@ struct BatchInst {
     int tab;         // table set index for this R
     int W;           // strip width
     int nstrips;
+    int range;       // smoothness indicators in their own scale (kVarRange)
 };
 
 struct BatchSeg {
@@ -52,7 +53,8 @@ constexpr size_t batch_smem_bytes()
 }
 
 // 512 (FP32) or 256 (FP64) resident threads per SM at most 128 / 255 registers each
-// VAR: 0, or kVarFlux for FP32 batches with an HLL or HLLC member; SPEC: the stage
+// VAR: 0, kVarFlux for FP32 batches with an HLL or HLLC member, or that with kVarRange where some member needs
+// it (the others keep the arithmetic they have alone); SPEC: the stage
 template <typename T, int NT, int VAR, int SPEC>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
     batch_stage_kernel(const BatchInst<T> *__restrict__ inst, const BatchSeg *__restrict__ segs,
@@ -67,7 +69,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
     // keeps them out of the registers the face evaluation needs
     __shared__ StageArgs<T> sa;
     __shared__ BatchSeg ssg;
-    __shared__ int sR, stab;
+    __shared__ int sR, stab, srange;
     __shared__ T sdt;
     const int k0 = cta_start[blockIdx.x], k1 = cta_start[blockIdx.x + 1];
     for (int k = k0; k < k1; ++k) {
@@ -131,6 +133,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
             ssg = sg;
             sR = I.R;
             stab = I.tab;
+            srange = I.range;
             sdt = (T)dt_dev[sg.inst];
         }
         __syncthreads();
@@ -141,11 +144,16 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 512 : 256) / NT)
         // spills with all three radii in one kernel); FP64 keeps the one-site loop, whose smaller
         // code spills less at 255 registers
         constexpr bool kOneSite = sizeof(T) == 8;
-        switch (sR) {
-        case 1: stage2d_segment<T, 1, NT, 4, VAR, kOneSite, SPEC>(sa, bt.t1[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
-        case 2: stage2d_segment<T, 2, NT, 4, VAR, kOneSite, SPEC>(sa, bt.t2[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
-        default: stage2d_segment<T, 3, NT, 4, VAR, kOneSite, SPEC>(sa, bt.t3[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
-        }
+        auto run = [&](auto var) {
+            constexpr int V = decltype(var)::value;
+            switch (sR) {
+            case 1: stage2d_segment<T, 1, NT, 4, V, kOneSite, SPEC>(sa, bt.t1[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+            case 2: stage2d_segment<T, 2, NT, 4, V, kOneSite, SPEC>(sa, bt.t2[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+            default: stage2d_segment<T, 3, NT, 4, V, kOneSite, SPEC>(sa, bt.t3[tab], sg.strip, sg.y0, sg.y1, smem, dt, rmx, rmy, ph); break;
+            }
+        };
+        if ((VAR & kVarRange) != 0 && !srange) run(std::integral_constant<int, VAR & ~kVarRange>());
+        else run(std::integral_constant<int, VAR>());
         // the segment ends with a barrier, so thread 0 may overwrite the shared arguments
     }
     if (__any_sync(0xffffffffu, !ph.good()) && (threadIdx.x & 31) == 0) atomicOr(flags, 1);

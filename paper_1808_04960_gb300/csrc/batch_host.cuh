@@ -106,13 +106,15 @@ inline bool read_tune_cache(const char *path, unsigned long long sig, BatchTiles
     return found;
 }
 
-// The batch kernel of a block size and stage, for batches of local Lax-Friedrichs members only or of any face flux.
+// The batch kernel of a block size and stage, for batches of local Lax-Friedrichs members only, of any face flux, or
+// also with members whose smoothness indicators keep their own scale.
 template <typename T, int NT, int SPEC>
 auto batch_kernel(const gpweno_plan_s *b)
 {
     auto kern = batch_stage_kernel<T, NT, 0, SPEC>;
     if constexpr (std::is_same<T, float>::value) {
         if (b->batch_riemann) kern = batch_stage_kernel<T, NT, kVarFlux, SPEC>;
+        if (b->batch_range) kern = batch_stage_kernel<T, NT, kVarFlux | kVarRange, SPEC>;
     }
     return kern;
 }
@@ -154,7 +156,11 @@ gpweno_status build_batch_T(gpweno_plan b)
     std::memset(&bt, 0, sizeof(bt));
     std::vector<gpweno_plan> reps[4];
     b->member_tab.assign(n, 0);
-    for (const gpweno_plan p : b->members) b->batch_riemann = b->batch_riemann || p->opts.flux_form != 0;
+    auto in_range = [](const gpweno_plan_s *p) { return std::is_same<T, double>::value || unit_scale_fits(p); };
+    for (const gpweno_plan p : b->members) {
+        b->batch_riemann = b->batch_riemann || p->opts.flux_form != 0;
+        b->batch_range = b->batch_range || !in_range(p);
+    }
     for (int k = 0; k < n; ++k) {
         gpweno_plan p = b->members[k];
         auto &rv = reps[p->R];
@@ -172,9 +178,9 @@ gpweno_status build_batch_T(gpweno_plan b)
             }
             idx = (int)rv.size();
             rv.push_back(p);
-            if (p->R == 1) bt.t1[idx] = make_tables<T, 1>(p);
-            if (p->R == 2) bt.t2[idx] = make_tables<T, 2>(p);
-            if (p->R == 3) bt.t3[idx] = make_tables<T, 3>(p);
+            if (p->R == 1) bt.t1[idx] = make_tables<T, 1, 0>(p);
+            if (p->R == 2) bt.t2[idx] = in_range(p) ? make_tables<T, 2, 0>(p) : make_tables<T, 2, kVarRange>(p);
+            if (p->R == 3) bt.t3[idx] = in_range(p) ? make_tables<T, 3, 0>(p) : make_tables<T, 3, kVarRange>(p);
         }
         b->member_tab[k] = idx;
     }
@@ -271,6 +277,7 @@ gpweno_status build_batch_T(gpweno_plan b)
         d.tab = b->member_tab[k];
         d.W = info[k].W;
         d.nstrips = info[k].nstrips;
+        d.range = !in_range(p);
     }
     b->batch_last_ptrs.assign(2 * n, nullptr);
     return GPWENO_OK;

@@ -3,6 +3,7 @@
 #pragma once
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 
 #include "list.cuh"
 #include "plan.h"
@@ -53,7 +54,7 @@ template <typename T>
 constexpr int kNTxy = sizeof(T) == 4 ? 128 : 256;
 constexpr int kNT1D = 128;
 
-template <typename T, int R>
+template <typename T, int R, int VAR>
 FaceTables<T, R> make_tables(const gpweno_plan_s *p)
 {
     FaceTables<T, R> t;
@@ -68,18 +69,17 @@ FaceTables<T, R> make_tables(const gpweno_plan_s *p)
         t.gl[m] = (T)(g.gl[m] / g.gl[UL]);
         t.gr[m] = (T)(g.gr[m] / g.gr[UR - 1]);
     }
-    const double a1 = g.fa;   // the scale of the smoothness indicators: the first difference's coefficient
-    t.A = (T)(g.fA / a1);
-    t.B = (T)(g.fB / a1);
-    t.D = (T)(g.fD / a1);
-    t.kb = (T)(g.fkb / a1);
-    t.kd = (T)(g.fkd / a1);
-    t.pA = (T)(g.fpA / a1);
-    t.pD = (T)(g.fpD / a1);
-    // eps in that scale; FP32: at least the floor, in the scaled and in the unscaled indicators, so that
-    // (eps + beta)^-2 stays in range
-    const double scale = 1.0 / (a1 * a1);
-    t.eps = (T)std::max(p->opts.eps * scale, (double)Num<T>::kEpsFloor * std::max(scale, 1.0));
+    const double unit = kUnitDifference<T, R, VAR> ? g.fa : 1.0;   // the scale of the smoothness indicators
+    t.A = (T)(g.fA / unit);
+    t.B = (T)(g.fB / unit);
+    t.D = (T)(g.fD / unit);
+    t.a = (T)(g.fa / unit);
+    t.kb = (T)(g.fkb / unit);
+    t.kd = (T)(g.fkd / unit);
+    t.pA = (T)(g.fpA / unit);
+    t.pD = (T)(g.fpD / unit);
+    // eps in that scale; FP32: at least the floor, so that (eps + beta)^-2 stays in range
+    t.eps = (T)(std::max(p->opts.eps, (double)Num<T>::kEpsFloor) / (unit * unit));
     t.gm1 = (T)(p->gamma - 1.0);
     t.igm1 = (T)(1.0 / (p->gamma - 1.0));
     t.hgm1 = (T)(0.5 * (p->gamma - 1.0));
@@ -87,6 +87,25 @@ FaceTables<T, R> make_tables(const gpweno_plan_s *p)
     t.p = p->opts.p;
     t.flux = p->opts.flux_form;
     return t;
+}
+
+// Whether an FP32 plan's weights stay in range in the scale of kUnitDifference: the floor of eps + beta becomes
+// floor / a^2, the largest weight (a^2 / floor)^p and the largest sum of weights that times the sum of the linear weights
+// over their unit, which has to stay below 2^126 for its reciprocal to be a normal number.  (Where a weight is
+// that large the data, and so the predictions summed with it, are below 1e-8.)  a^2 <= 6.3 at R = 2 and 5.1 at
+// R = 3 for the default eps and long l, that is sigma <= 4.9 and 6.5 dx; any sigma for p = 1.
+inline bool unit_scale_fits(const gpweno_plan_s *p)
+{
+    if (p->R == 1) return true;   // no kernel takes it
+    const GpTables &g = p->tab;
+    const int ul = p->R == 2 ? kUnitL<2> : kUnitL<3>, ur = p->R == 2 ? kUnitR<2> : kUnitR<3>;
+    double l = 0.0, r = 0.0;
+    for (int m = 0; m <= p->R; ++m) {
+        l += std::fabs(g.gl[m] / g.gl[ul]);
+        r += std::fabs(g.gr[m] / g.gr[ur - 1]);
+    }
+    const double x = g.fa * g.fa / std::max(p->opts.eps, (double)Num<float>::kEpsFloor);
+    return (p->opts.p == 2 ? x * x : x) * std::max(l, r) <= 8.5e37;
 }
 
 // Tables of a scheme variant: GP-AO adds its own on top of the GP-WENO ones.
@@ -98,7 +117,7 @@ TablesFor<T, R, VAR> make_tables_var(const gpweno_plan_s *p)
         constexpr int NH = AT::NH, NL = AT::NL;
         AT t;
         std::memset(&t, 0, sizeof(t));
-        static_cast<FaceTables<T, R> &>(t) = make_tables<T, R>(p);
+        static_cast<FaceTables<T, R> &>(t) = make_tables<T, R, VAR>(p);
         const AoTables &a = p->ao;
         for (int j = 0; j < NH; ++j) {
             t.whl[j] = (T)a.w_hi_l[j];
@@ -143,7 +162,7 @@ TablesFor<T, R, VAR> make_tables_var(const gpweno_plan_s *p)
         t.g3[1] = (T)((1.0 - gh) * gl);
         return t;
     } else {
-        return make_tables<T, R>(p);
+        return make_tables<T, R, VAR>(p);
     }
 }
 
@@ -490,7 +509,7 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
         // x1.05 at 768^2, x1.017 at 1024^2; R = 1 x1.14 at 700 x 640, x1.05 at 777 x 613; R = 3 x1.10 at
         // 777 x 613, x1.05 at 1024 x 512, x1.03 at 1501 x 1100, x1.016 at 2048^2 (HLLC x1.013, x1.005).  Not
         // taken where it lost: R = 2 at 1536^2 (x0.995) and 4096^2 (x0.98), R = 1 at 1024^2 (x0.98).
-        constexpr bool kHasWide = std::is_same<T, float>::value && (VAR & ~(kVarSlab | kVarFlux)) == 0;
+        constexpr bool kHasWide = std::is_same<T, float>::value && (VAR & ~(kVarSlab | kVarFlux | kVarRange)) == 0;
         if constexpr (kHasWide) {
             const int slots4 = 512 / NT * p->num_sms;
             const Schedule s4 = schedule2d(a.n[0], a.n[1], NT, slots4);

@@ -164,6 +164,27 @@ struct Physical<double> {
     __device__ __forceinline__ bool good() const { return ok; }
 };
 
+// Scheme variants chosen at compile time: bit 0 the non-zero-mean smoothness
+// indicators, bit 1 the FD-Flux form, bit 2 GP-AO; bit 3 is not a scheme change
+// but a grid with an external (halo) side, whose loaders read ghost layers from
+// halo buffers -- a separate instantiation so that the loaders of the others stay
+// as they are.
+// Bit 4 (FP32): HLL and HLLC face fluxes; kernels without it are compiled for the local Lax-Friedrichs
+// flux alone (2 % per step at 1024^2, 3 % in batches, 3-4 % in the GP-AO kernels).  FP64 kernels hold all three.
+constexpr int kVarMean = 1, kVarFdFlux = 2, kVarAo = 4, kVarSlab = 8, kVarFlux = 16;
+// Bit 5 (FP32): smoothness indicators in their own scale for plans whose weights leave the FP32 range in the one
+// that the other kernels take (kUnitDifference, unit_scale_fits): sigma beyond about 5 (R = 2) and 6 dx (R = 3).
+constexpr int kVarRange = 32;
+
+// Whether the smoothness indicators are divided by the square of the last form's coefficient a (beta_weight), which
+// saves an instruction per window: FP32 step of 4096^2 R = 2 2288 -> 2220 us, of 512^3 R = 3 50.7 -> 50.0 ms, HLLC R = 3
+// 397 -> 387 us; none at R = 1 (777 x 613 25.3 us both ways).  The floor of eps + beta is divided alike (a = 1.6 at R = 2,
+// 1.1 at R = 3 for sigma = 3 dx, growing with sigma), so (eps + beta)^-p grows by a^2p.  FP32 keeps the indicators'
+// own scale where that leaves the range: in the kVarRange kernels; at R = 1 (a = 3 already); and
+// with the centre's mean, whose weighted sums hold predictions of any size also where beta is at its floor.
+template <typename T, int R, int VAR>
+constexpr bool kUnitDifference = sizeof(T) == 8 || (R > 1 && (VAR & (kVarRange | kVarMean)) == 0);
+
 // Weight tables of one plan in the arithmetic type.  Passed by value as a
 // kernel parameter so every (warp-uniform) table read is a constant-bank
 // operand.
@@ -178,10 +199,10 @@ struct FaceTables {
     T gl[R + 1];          // linear weights of the left state (windows 0..R) over that of window kUnitL
     T gr[R + 1];          // linear weights of the right state (windows 1..R+1) over that of window kUnitR
     // smoothness factor of K_m(sigma), K_m^-1 = sum of squares of five forms of the window's sums
-    // f_j + f_{R-j} and differences f_{R-j} - f_j, divided by the first difference's coefficient
-    // (see window_factors): outer sum (A, B with the inner one or the middle cell), inner (D),
-    // outer difference (1, kb with the inner one), inner (kd)
-    T A, B, D, kb, kd;
+    // f_j + f_{R-j} and differences f_{R-j} - f_j (see window_factors): outer sum (A, B with the inner one or the
+    // middle cell), inner (D), differences (kb the outer, kd the inner one), outer difference (a); divided by a where
+    // the kernel takes it for 1, see kUnitDifference
+    T A, B, D, a, kb, kd;
     T pA, pD;             // row sums of the two symmetric forms
     T eps;                // WENO epsilon in the same scale (FP32: at least the floor of Num<T>)
     T gamma;              // ratio of specific heats
@@ -447,9 +468,9 @@ __device__ __forceinline__ CellPart<T, NC> cell_part(const T (&U)[NC], const Tab
 // orthogonal basis) over the window f[w..w+R] of data f_j - shift = d_j + (f_c - shift), with
 // d_R = 0 (relative to the face's cell s).  pA, pD = (f_c - shift) times the row sums of the two
 // symmetric forms, supplied by the caller (the differences' row sums vanish).  Triangular forms
-// (window_factors) and the unit coefficient of the first difference save 2 (R = 2) and 3 (R = 3)
-// of 10 and 16 instructions per window against the eigenvector rows.
-template <typename T, int R, typename V, int NS>
+// (window_factors) save 1 (R = 2) and 2 (R = 3) of 10 and 16 instructions per window against the eigenvector
+// rows, and UNIT one more: the scale in which the coefficient a of the last form is 1 (kUnitDifference).
+template <typename T, int R, bool UNIT, typename V, int NS>
 __device__ __forceinline__ V beta_weight(const FaceTables<T, R> &tb, const V (&d)[NS], int w, V pA, V pD)
 {
     // sum and difference of the window's cells j and R-j; `flip` picks the sign of all differences of a
@@ -464,7 +485,8 @@ __device__ __forceinline__ V beta_weight(const FaceTables<T, R> &tb, const V (&d
         return lo == R ? d[hi] : vsub(d[hi], d[lo]);
     };
     V beta = vcast(tb.eps, V());   // (eps + beta), accumulated from eps
-    V s = vfma(tb.A, sum(0), pA), k = diff(0);
+    V s = vfma(tb.A, sum(0), pA);
+    const V t = diff(0), k = UNIT ? t : vmul(tb.a, t);
     if constexpr (R == 2) {
         V m = pD;
         if (w + 1 != R) {
@@ -476,8 +498,7 @@ __device__ __forceinline__ V beta_weight(const FaceTables<T, R> &tb, const V (&d
     if constexpr (R == 3) {
         const V si = sum(1), ki = diff(1);
         s = vfma(tb.B, si, s);
-        const V m = vfma(tb.D, si, pD), n = vmul(tb.kd, ki);
-        k = vfma(tb.kb, ki, k);
+        const V m = vfma(tb.D, si, pD), n = vfma(tb.kb, t, vmul(tb.kd, ki));
         beta = vfma(m, m, beta);
         beta = vfma(n, n, beta);
     }
@@ -494,7 +515,7 @@ __device__ __forceinline__ V beta_weight(const FaceTables<T, R> &tb, const V (&d
 // both sides, and omega_m ~ gamma_m x_k with x_k = (eps + beta_k)^-p (Eq. weights); sum_m omega_m = 1
 // is used exactly.  With the zero mean x_k and x_k q_k are shared too.  MEAN: the left side's windows
 // shift by its centre, cell s (no shift), the right side's by cell s+1 (shift d_{R+1}).
-template <typename T, int R, bool MEAN, typename V, int NS>
+template <typename T, int R, bool MEAN, bool UNIT, typename V, int NS>
 __device__ __forceinline__ void weno_states(const FaceTables<T, R> &tb, const V (&d)[NS], V fc, V &qL, V &qR)
 {
     constexpr int UL = kUnitL<R>, UR = kUnitR<R>;
@@ -509,12 +530,12 @@ __device__ __forceinline__ void weno_states(const FaceTables<T, R> &tb, const V 
         for (int j = 0; j <= R; ++j)
             if (k + j != R) q = vfma(tb.w[k][j], d[k + j], q);
         if (k <= R) {
-            xl = beta_weight<T, R>(tb, d, k, lA, lD);
+            xl = beta_weight<T, R, UNIT>(tb, d, k, lA, lD);
             tl = vmul(xl, q);
         }
         if (k > 0) {
             if (MEAN || k > R) {
-                xr = beta_weight<T, R>(tb, d, k, rA, rD);
+                xr = beta_weight<T, R, UNIT>(tb, d, k, rA, rD);
                 tr = vmul(xr, q);
             } else {
                 xr = xl;
@@ -794,12 +815,13 @@ __device__ __forceinline__ void face_flux(const FaceRoe<T, NC> &f, const Tables 
 // measured per step against the form without them: FP32 1024^2 R = 2 232 -> 205 us, 4096^2
 // 2848 -> 2460 us, 3D 512^3 R = 3 63.1 -> 53.4 ms; FP64 512^2 R = 2 3086 -> 2702 us.
 // LF: local Lax-Friedrichs only (tb.flux is not read).  P5: five fields packed in FP32.
-template <typename T, int NC, int R, bool MEAN = false, bool AO = false, bool LF = false, bool P5 = false>
+template <typename T, int NC, int R, int VAR, bool LF, bool P5>
 __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
                                          T (&M)[NC], Physical<T> &ph)
 {
     constexpr int NS = 2 * R + 2;
     constexpr int E = NC - 1;
+    constexpr bool MEAN = (VAR & kVarMean) != 0, AO = (VAR & kVarAo) != 0;
     const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
     const T igm1 = tb.igm1;
     const PrimRef<T, NC> &ref = f.ref;
@@ -832,7 +854,7 @@ __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const Fac
 #pragma unroll
             for (int j = 0; j < NS; ++j)
                 d[j] = (j == R) ? f2(0.0f) : make_float2(f.lrow(k0, dV[j]), f.lrow(k1, dV[j]));
-            weno_states<T, R, MEAN>(tb, d, fc, qL, qR);
+            weno_states<T, R, MEAN, kUnitDifference<T, R, VAR>>(tb, d, fc, qL, qR);
             dqL[k0] = qL.x;
             dqR[k0] = qR.x;
             dqL[k1] = qL.y;
@@ -851,7 +873,7 @@ __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const Fac
             dqL[kk] = ao_side<T, R, NS, false, MEAN>(ta, d, fc);                 // q_L - L V_s
             dqR[kk] = ao_side<T, R, NS, true, MEAN>(ta, d, fc) - d[R + 1];      // q_R - L V_{s+1}
         } else {
-            weno_states<T, R, MEAN>(tb, d, fc, dqL[kk], dqR[kk]);
+            weno_states<T, R, MEAN, kUnitDifference<T, R, VAR>>(tb, d, fc, dqL[kk], dqR[kk]);
         }
     }
 
@@ -873,7 +895,7 @@ __device__ __forceinline__ void face_rel(const T (&st)[2 * R + 2][NC], const Fac
 // Sum of the two reconstructed parts of one field (or two) of the FD-Flux form, relative to cell s:
 // the left part from p (relative to its cell-s value fcp) on windows 0..R, the right part from m
 // (fcm) on windows 1..R+1.  Zero mean: shifts fcp and fcm; MEAN: centres cell s and cell s+1.
-template <typename T, int R, bool MEAN, typename V, int NS>
+template <typename T, int R, bool MEAN, bool UNIT, typename V, int NS>
 __device__ __forceinline__ V fdf_state(const FaceTables<T, R> &tb, const V (&p)[NS], const V (&m)[NS], V fcp, V fcm)
 {
     constexpr int UL = kUnitL<R>, UR = kUnitR<R>;
@@ -885,7 +907,7 @@ __device__ __forceinline__ V fdf_state(const FaceTables<T, R> &tb, const V (&p)[
 #pragma unroll
         for (int j = 0; j <= R; ++j)
             if (k + j != R) q = vfma(tb.w[k][j], d[k + j], q);
-        x = beta_weight<T, R>(tb, d, k, sA, sD);
+        x = beta_weight<T, R, UNIT>(tb, d, k, sA, sD);
         return vmul(x, q);
     };
     V denL, denR, x;
@@ -920,11 +942,12 @@ __device__ __forceinline__ V fdf_state(const FaceTables<T, R> &tb, const V (&p)[
 // values, each reconstructed part minus g+-_s is
 // sum_m omega_m (w_m . d_m + (sum_j w_mj - 1) g+-_s), and g+_s + g-_s = l(F_s)
 // projects back to F(U_s).  Requires physical states in `ph`.
-template <typename T, int NC, int R, bool MEAN = false>
+template <typename T, int NC, int R, int VAR>
 __device__ __forceinline__ void face_fdf(const T (&st)[2 * R + 2][NC], const FaceTables<T, R> &tb, T (&A)[NC],
                                          T (&M)[NC], Physical<T> &ph)
 {
     constexpr int NS = 2 * R + 2, E = NC - 1, NV = NC - 2;
+    constexpr bool MEAN = (VAR & kVarMean) != 0;
     const FaceRoe<T, NC> f = face_roe<T, NC>(st[R], st[R + 1], tb);
     T vel[NV], q2 = T(0), B[NC];
 #pragma unroll
@@ -1015,7 +1038,7 @@ __device__ __forceinline__ void face_fdf(const T (&st)[2 * R + 2][NC], const Fac
                 p2[j] = make_float2(dp[k0][j], dp[k1][j]);
                 m2[j] = make_float2(dm[k0][j], dm[k1][j]);
             }
-            const float2 q = fdf_state<T, R, MEAN>(tb, p2, m2, vmul(0.5f, vfma(alpha, lvs, lgs)),
+            const float2 q = fdf_state<T, R, MEAN, kUnitDifference<T, R, VAR>>(tb, p2, m2, vmul(0.5f, vfma(alpha, lvs, lgs)),
                                                    vmul(0.5f, vfma(-alpha, lvs, lgs)));
             dq[k0] = q.x;
             dq[k1] = q.y;
@@ -1024,7 +1047,7 @@ __device__ __forceinline__ void face_fdf(const T (&st)[2 * R + 2][NC], const Fac
 #pragma unroll
     for (int kk = kScalarFrom; kk < NC; ++kk) {
         const T lgs = f.lrow(kk, JFs), lvs = f.lrow(kk, JUs);
-        dq[kk] = fdf_state<T, R, MEAN>(tb, dp[kk], dm[kk], T(0.5) * fma(alpha, lvs, lgs),
+        dq[kk] = fdf_state<T, R, MEAN, kUnitDifference<T, R, VAR>>(tb, dp[kk], dm[kk], T(0.5) * fma(alpha, lvs, lgs),
                                        T(0.5) * fma(-alpha, lvs, lgs));
     }
 
@@ -1047,15 +1070,6 @@ __device__ __forceinline__ void face_fdf(const T (&st)[2 * R + 2][NC], const Fac
     for (int a = 0; a < NC; ++a) M[a] = A[a] - B[a];
 }
 
-// Scheme variants chosen at compile time: bit 0 the non-zero-mean smoothness
-// indicators, bit 1 the FD-Flux form, bit 2 GP-AO; bit 3 is not a scheme change
-// but a grid with an external (halo) side, whose loaders read ghost layers from
-// halo buffers -- a separate instantiation so that the loaders of the others stay
-// as they are.
-// Bit 4 (FP32): HLL and HLLC face fluxes; kernels without it are compiled for the local Lax-Friedrichs
-// flux alone (2 % per step at 1024^2, 3 % in batches, 3-4 % in the GP-AO kernels).  FP64 kernels hold all three.
-constexpr int kVarMean = 1, kVarFdFlux = 2, kVarAo = 4, kVarSlab = 8, kVarFlux = 16;
-
 // Kernel parameter type of a variant's tables.
 template <typename T, int R, int VAR>
 using TablesFor = typename std::conditional<(VAR & kVarAo) != 0, AoFaceTables<T, R>, FaceTables<T, R>>::type;
@@ -1065,8 +1079,8 @@ __device__ __forceinline__ void face_eval(const T (&st)[2 * R + 2][NC], const Fa
                                           T (&M)[NC], Physical<T> &ph)
 {
     constexpr bool kLf = std::is_same<T, float>::value && (VAR & kVarFlux) == 0;
-    if constexpr ((VAR & kVarFdFlux) != 0) face_fdf<T, NC, R, (VAR & kVarMean) != 0>(st, tb, A, M, ph);
-    else face_rel<T, NC, R, (VAR & kVarMean) != 0, (VAR & kVarAo) != 0, kLf, P5>(st, tb, A, M, ph);
+    if constexpr ((VAR & kVarFdFlux) != 0) face_fdf<T, NC, R, VAR>(st, tb, A, M, ph);
+    else face_rel<T, NC, R, VAR, kLf, P5>(st, tb, A, M, ph);
 }
 
 // Weights of the corrected-flux difference: with the face-flux correction

@@ -518,15 +518,17 @@ bool window_factors(dd qs, int S, GpTables *out)
             }
         return v;
     };
-    const dd A = sqrt_dd(form(0, 0, 1.0)), a = sqrt_dd(form(0, 0, -1.0));
+    const dd A = sqrt_dd(form(0, 0, 1.0));
+    dd a = sqrt_dd(form(0, 0, -1.0));
     dd B = make(0.0), D = make(0.0), kb = make(0.0), kd = make(0.0);
     if (S > 2) {
         B = div(form(0, 1, 1.0), A);
         D = sqrt_dd(sub(form(1, 1, 1.0), mul(B, B)));
     }
-    if (S > 3) {
-        kb = div(form(0, 1, -1.0), a);
-        kd = sqrt_dd(sub(form(1, 1, -1.0), mul(kb, kb)));
+    if (S > 3) {   // the inner difference first, so that the outer one is left alone in the last form
+        kd = sqrt_dd(form(1, 1, -1.0));
+        kb = div(form(0, 1, -1.0), kd);
+        a = sqrt_dd(sub(form(0, 0, -1.0), mul(kb, kb)));
     }
     const double inner = S == 3 ? 1.0 : 2.0;   // cells that a unit of s_1 spans
     out->fA = to_d(A);

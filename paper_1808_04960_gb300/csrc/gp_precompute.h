@@ -23,7 +23,7 @@ struct GpTables {
     double lambda[kMaxS];
     // The same quadratic form in the window's sums s_j = f_j + f_{R-j} (outer first; the middle cell
     // itself for odd R+1) and differences t_j = f_{R-j} - f_j, each part factored triangularly:
-    //   f^T K_m(sigma)^-1 f = (fA s_0 + fB s_1)^2 + (fD s_1)^2 + (fa t_0 + fkb t_1)^2 + (fkd t_1)^2
+    //   f^T K_m(sigma)^-1 f = (fA s_0 + fB s_1)^2 + (fD s_1)^2 + (fkb t_0 + fkd t_1)^2 + (fa t_0)^2
     // (K_m is persymmetric, so sums and differences do not mix), with the row sums fpA, fpD of the
     // first two forms over the window's cells.
     double fA, fB, fD, fa, fkb, fkd, fpA, fpD;

@@ -70,6 +70,7 @@ struct gpweno_plan_s {
     int batch_oversub = 1;                  // CTA shares per resident slot
     int batch_grid = 0;                     // CTAs per launch
     bool batch_riemann = false;             // some member's face flux is HLL or HLLC
+    bool batch_range = false;               // some member's smoothness indicators keep their own scale (FP32)
     int batch_nseg = 0;                     // segments in the schedule
     unsigned long long batch_signature = 0; // hash of the instance list (tuning-cache key)
     std::string batch_tune_path;            // tuning cache file (may be empty)
@@ -157,6 +158,10 @@ gpweno_status launch_stage_f32_var17(gpweno_plan p, const StageIO &io, cudaStrea
 gpweno_status launch_stage_f32_var20(gpweno_plan p, const StageIO &io, cudaStream_t st);
 gpweno_status launch_stage_f32_var21(gpweno_plan p, const StageIO &io, cudaStream_t st);
 gpweno_status launch_stage_f32_var24(gpweno_plan p, const StageIO &io, cudaStream_t st);
+// FP32 smoothness indicators in their own scale: kVarRange = 32 with FD-Flux, any face flux, and that on slabs
+gpweno_status launch_stage_f32_var34(gpweno_plan p, const StageIO &io, cudaStream_t st);
+gpweno_status launch_stage_f32_var48(gpweno_plan p, const StageIO &io, cudaStream_t st);
+gpweno_status launch_stage_f32_var56(gpweno_plan p, const StageIO &io, cudaStream_t st);
 // tiles of an FP32 2D plan (none for larger grids)
 Tile2D choose_tile_f32(const gpweno_plan_s *p);
 // layers per band and bytes of an FP64 plan's face workspace (zero bytes: none)

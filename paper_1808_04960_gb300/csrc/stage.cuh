@@ -955,7 +955,7 @@ __global__ void __launch_bounds__(96) stage1d_split_kernel(StageArgs<T> a, Table
             d[j] = j == R ? T(0) : (k == 0 ? f.lrow(0, dV[j]) : (k == 1 ? f.lrow(1, dV[j]) : f.lrow(E, dV[j])));
         const T fc = k == 0 ? f.lrow(0, f.Vs) : (k == 1 ? f.lrow(1, f.Vs) : f.lrow(E, f.Vs));
         T qL, qR;
-        weno_states<T, R, MEAN>(tb, d, fc, qL, qR);
+        weno_states<T, R, MEAN, kUnitDifference<T, R, VAR>>(tb, d, fc, qL, qR);
         q[0][k][lane] = qL;
         q[1][k][lane] = qR;
 #pragma unroll
