@@ -80,6 +80,8 @@ FaceTables<T, R> make_tables(const gpweno_plan_s *p)
     t.pD = (T)(g.fpD / unit);
     // eps in that scale; FP32: at least the floor, so that (eps + beta)^-2 stays in range
     t.eps = (T)(std::max(p->opts.eps, (double)Num<T>::kEpsFloor) / (unit * unit));
+    // FP64: an eps whose eps^-p is finite stays so in that scale (down to it beta is lost against no data above 1e-70)
+    if (std::is_same<T, double>::value) t.eps = (T)std::max((double)t.eps, p->opts.p == 2 ? 1e-150 : 1e-300);
     t.gm1 = (T)(p->gamma - 1.0);
     t.igm1 = (T)(1.0 / (p->gamma - 1.0));
     t.hgm1 = (T)(0.5 * (p->gamma - 1.0));

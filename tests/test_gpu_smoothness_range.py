@@ -52,6 +52,23 @@ def test_f32_jump_of_small_data(R, sigma, shape, opts):
     assert err <= 1e-3
 
 
+@pytest.mark.parametrize("R,sigma,eps,p", [(1, 12.0, 1e-152, 2), (2, 40.0, 1e-152, 2), (3, 12.0, 1e-153, 2),
+                                           (1, 900.0, 1e-303, 1), (3, 3.0, 1e-36, 2)])
+def test_f64_smallest_eps(R, sigma, eps, p):
+    """FP64 weights of data whose beta is exactly zero (v = 0 beside the jump) stay finite for every eps whose own
+    (eps)^-p is; against the oracle, 1e-10 of the largest value, the bound of the FP64 parity tests."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    oracle.build()
+    U, meta = shear_jump((24, 64), 0.1)
+    want = oracle.Oracle(U.shape[1:], meta["dx"], meta["bc"], R=R, sigma_over_dx=sigma, eps=eps, p=p).rhs(U)
+    plan = gpweno.Plan(R, 12.0, U.shape[1:], meta["dx"], meta["bc"], dtype="f64", sigma_over_dx=sigma, eps=eps, p=p)
+    got = plan.rhs(torch.from_numpy(U).cuda()).cpu().numpy()
+    assert plan.flags() == 0 and np.isfinite(got).all()
+    assert np.abs(got - want).max() <= 1e-10 * np.abs(want).max()
+
+
 @pytest.mark.parametrize("fluxes", [("lf", "lf"), ("hllc", "lf")])
 def test_batch_of_both_scales(fluxes):
     """sigma = 3 and 12 dx take different kernels alone; a batch of both equals them bit for bit."""
