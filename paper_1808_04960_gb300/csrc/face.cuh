@@ -78,8 +78,8 @@ struct Num<float> {
 // and take one third-order step of the binomial series (Householder's method of order two):
 //   1/a       = x / (1 - e) = x (1 + e + e^2 + ...),             e = 1 - a x,    |e| <= ~2^-19
 //   a^(-1/2)  = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...),  e = 1 - a y^2
-// with remainders below 2^-56: results within one unit in the last place, in 3 and 5 FP64
-// instructions in place of an IEEE division or square root plus division.  Order tests and maxima
+// with remainders below 2^-55: results within one unit in the last place, in 3 and 5 FP64
+// instructions (the square root in 6) in place of an IEEE division or square root plus division.  Order tests and maxima
 // run on the bit patterns in the integer units.  Measured per RK3 step: 512^2 R = 2 3629 -> 3086 us,
 // 128^2 R = 3 3042 -> 2748 us; one 3D right-hand side of 70x61x45 2870 -> 2421 us.  Arguments are normal positive numbers
 // (eps + beta, densities, sums of weights); zero, infinity or NaN give NaN, which the
@@ -100,7 +100,16 @@ struct Num<double> {
         const double e = fma(-(a * y), y, 1.0);
         return fma(y * e, fma(0.375, e, 0.5), y);
     }
-    static __device__ __forceinline__ double sqrt(double a) { return __dmul_rn(a, rsqrt(a)); }
+    // s (1 - E)^(-1/2) = s (1 + E/2 + 3 E^2/8 + ...) with s = a y and E = (a - s^2) / a, whose numerator is exact: the same
+    // six instructions as a times rsqrt(a), which would round twice more (1.6 units in the last place; this: 0.52)
+    static __device__ __forceinline__ double sqrt(double a)
+    {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+        const double s = __dmul_rn(a, y);
+        const double t = __dmul_rn(fma(-s, s, a), y);   // s E
+        return fma(t, fma(0.375, fma(-s, y, 1.0), 0.5), s);
+    }
     // IEEE forms, zero and infinity included: once per cell, in the CFL rates
     static __device__ __forceinline__ double rcp_ieee(double x) { return 1.0 / x; }
     static __device__ __forceinline__ double sqrt_ieee(double x) { return ::sqrt(x); }
