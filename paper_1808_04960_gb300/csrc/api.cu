@@ -633,7 +633,7 @@ gpweno_status gpweno_flags(gpweno_plan p, int *nonphysical)
     unsigned long long f = 0;
     GPW_CHECK(cudaMemcpy(&f, p->ws + 3, sizeof(f), cudaMemcpyDeviceToHost), "gpweno_flags: read");
     GPW_CHECK(cudaMemset(p->ws + 3, 0, sizeof(f)), "gpweno_flags: clear");
-    *nonphysical = (f & 1ull) ? 1 : 0;
+    *nonphysical = (int)f;
     return GPWENO_OK;
 }
 

@@ -48,6 +48,12 @@ void fake_device(int d) { g_device = d; }
 long fake_launches() { return g_launches; }
 long fake_lowered() { return g_lowered; }            // times a kernel's limit was set below an earlier value
 size_t fake_bytes() { return g_bytes; }              // device memory held
+void *fake_block(size_t bytes)                       // an allocation of that size
+{
+    for (const auto &b : g_blocks)
+        if (b.second.first == bytes) return const_cast<void *>(b.first);
+    return nullptr;
+}
 void fake_budget(size_t bytes) { g_budget = bytes; } // cudaMalloc fails beyond it
 void fake_hold() { g_hold = 1; }                     // the next residency query returns only after fake_release()
 int fake_held() { return g_held; }

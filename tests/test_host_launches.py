@@ -160,3 +160,18 @@ fake.fake_budget(fake.fake_bytes() + (1 << 20))
 p = plan((256, 256), 2, "f64")
 assert held(p) == 0
 """)
+
+
+def test_flags_return_every_bit(run):
+    """gpweno_flags returns the whole word: bits 1-11 are the bounds-checked build's access sites."""
+    run("""
+fake.fake_block.restype, fake.fake_block.argtypes = ctypes.c_void_p, [ctypes.c_size_t]
+p = plan((100, 100))
+word = ctypes.c_ulonglong.from_address(fake.fake_block(32) + 24)
+v = ctypes.c_int()
+for bits in (0, 1, 1 << 4, (1 << 11) | 1, 0xffe):
+    word.value = bits
+    for want in (bits, 0):
+        g._check(lib.gpweno_flags(p, ctypes.byref(v)))
+        assert v.value == want, (bits, v.value)
+""")
