@@ -58,6 +58,9 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
     os.makedirs(out_dir, exist_ok=True)
     nvcc = _nvcc()
     common = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
+    # nvcc compresses device code from about 10 MB per file on; decompressing it made the first HLLC or slab call of a
+    # process take 9.7 ms, against 1.3 as it is (the library grows from 143 to 200 MB)
+    common += ["--compress-mode=none"]
     if checked:
         common.append("-DGPWENO_CHECKED")
 
