@@ -192,11 +192,18 @@ template <int R, int VAR>
 constexpr int kTileThreads = R == 3 && (VAR & (kVarAo | kVarFdFlux)) != 0 ? 384 : kNTtile;
 
 // Strip marching's CTAs of eight rows per SM (the most it makes) below which an FP32 2D grid is tiled.  Measured
-// step times, marching / tiles, at 512^2 (2.1), 768^2 (4.4), 1024^2 (7.6) and 1500^2 (16): HLLC R = 2 108/60, 143/127,
-// 222/218, 421/451 us; FD-Flux R = 2 148/93, 200/192, 311/352, 595/789; GP-AO R = 2 169/81, 239/175, 370/303,
-// 708/646, R = 3 224/132, 372/308, 587/515, 1159/1141; right-hand side alone R = 1/2/3 at 777 x 613 32/36/47 and
-// 25/31/37, at 1024^2 52/64/84 and 51/61/75, at 1500^2 96/121/157 and 104/122/152.  Steps of the default scheme
-// end at two CTAs per SM, below 512^2: their schedule of strips is what gpweno_plan_schedule reports from there on.
+// times, marching / tiles, at 512^2 (2.1 CTAs per SM), 777 x 613 (3.5), 768^2 (4.4), 1000 x 900 (6.7), 1024^2 (7.6), 1500^2 (16):
+//   HLLC step  R = 1  84/53  94/94   111/103 152/164 168/189 312/397 us    R = 2 100/62  113/110 130/127 179/182 201/217 382/453
+//              R = 3 125/76  144/131 176/159 242/225 268/256 499/538
+//   FD-Flux    R = 1  95/59  108/103 123/115 170/178 192/202 367/427       R = 2 137/90  158/167 182/190 252/291 283/347 547/790
+//              R = 3 170/111 245/205 295/254 395/375 445/430 873/967
+//   GP-AO      R = 2 154/82  182/149 212/174 301/254 334/303 649/648       R = 3 203/131 303/238 359/297 518/438 580/504 1125/1097
+//   RHS alone  R = 1  23/16   27/29   31/31   43/45   47/53   84/107       R = 2  29/21   33/33   37/37   51/53   57/62  109/123
+//              R = 3  37/25   43/39   51/47   72/68   79/76  143/155
+// The lines were drawn with marching kernels that were 6 to 13 % slower (before they were compiled per stage), hence
+// within 7 % of break-even where they lie past it (R = 1 and FD-Flux R = 2 at 3.5).  Steps of the default scheme
+// (72/49, 88/57, 115/70 us at 512^2, 98/94, 116/117, 162/146 at 768^2, 146/170, 178/198, 247/235 at 1024^2) end at two CTAs
+// per SM, below 512^2, not by these times: their schedule of strips is what gpweno_plan_schedule reports from there on.
 template <int R, int VAR>
 constexpr int kTileLimit = (VAR & kVarAo) != 0 ? 16 : ((VAR & kVarFdFlux) != 0 && R == 2 ? 4 : (R == 1 ? 5 : (R == 2 ? 6 : 8)));
 constexpr int kTileLimitStep = 2, kTileLimitMost = 16;
@@ -316,7 +323,7 @@ gpweno_status launch_stage2d_spec(gpweno_plan p, StageArgs<T> a, const TablesFor
     auto kern = stage2d_kernel<T, R, NT, VAR, MINB, SPEC>;
     static Residency residency;   // per instantiation
     int occ;
-    // at most MINB: R = 1's three-CTA build needs 125 registers and would fit four times
+    // at most MINB: R = 1's three-CTA build needs 120 registers at most and would fit four times
     const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, MINB, "stage2d occupancy", occ);
     if (r != GPWENO_OK) return r;
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
@@ -503,7 +510,8 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             }
         }
         // FP32, default scheme (also with slab halos): the build for three CTAs per SM (more
-        // registers per thread: R = 2/3 140/159 instead of 128; R = 1 needs 125 either way) is faster where
+        // registers per thread: 120 to 134 at R = 2, 142 to 156 at R = 3 by stage, the four-CTA build's 128 being the
+        // limit there; R = 1 needs 108 to 120 either way) is faster where
         // the four-CTA schedule cannot fill four CTAs per SM (the grid is row-limited), and for
         // R = 2, whose four-CTA build is register-capped, where it leaves a CTA fewer than
         // kWideRows rows (three CTAs per SM: fewer, taller segments, fewer warm-up rows).
@@ -588,10 +596,10 @@ gpweno_status launch_stage_T(gpweno_plan p, const StageIO &io, cudaStream_t st)
     }
 }
 
-// Workspace of the FP64 face-list stages: layers per band and bytes, chosen at plan creation.  A band has at
-// least 24 layers (the five faces that neighbouring bands repeat then cost at most a fifth of one
-// direction) and up to 32 MiB, which keeps its face fluxes in L2; 32 MiB is 256 K cells in 2D, over fifty
-// warps of faces per SM.  Grids whose 24 layers need more than 1 GiB (3D from 420^2 per plane, 2D
+// Workspace of the FP64 face-list stages: layers per band and bytes, chosen at plan creation.  Bands are equal, of up
+// to 24 layers, or of more as far as 32 MiB go, which keeps their face fluxes in L2; equal means that a band has more than
+// half of that: five faces of every 24 (a fifth of one direction) are repeated by neighbouring bands at best, of 13
+// where 25 layers make two.  32 MiB is 256 K cells in 2D, over fifty warps of faces per SM.  Grids whose 24 layers need more than 1 GiB (3D from 420^2 per plane, 2D
 // from 300 K columns) keep the marching kernels.
 inline void size_face_workspace(gpweno_plan_s *p)
 {

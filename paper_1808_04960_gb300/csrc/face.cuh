@@ -221,7 +221,7 @@ struct FaceTables {
 };
 
 // Window whose linear weight is the unit of each side's weights: the one that is never small
-// against the others for any l/dx >= 1 (ratio at most 3.7), so the scaled sums stay in range.
+// against the others for any l/dx >= 1 (ratio at most 3.7, with FD-Flux 4.2), so the scaled sums stay in range.
 template <int R>
 constexpr int kUnitL = R == 2 ? 2 : 1;
 template <int R>

@@ -6,9 +6,9 @@
 // thread a face), and then updates its cells: two or three faces deep instead of twenty-one.  The price is
 // the five extra faces per tile row and column, (TX+5)/TX and (TY+5)/TY of the work, which is
 // why larger grids march.  choose_tile (dispatch.cuh) sizes the tiles for the SM count.
-// Measured on GB300 per step, R = 2 (marching -> tiles, equal bits): 256^2 61.8 -> 22.8 us, 384^2 71.7 -> 36.7,
-// 480^2 100.7 -> 50.4, 1000 x 200 77.7 -> 46.2; 64^2 55 -> 14 us (the launches).  At 2048^2 tiles lose:
-// 753 us against 643.
+// Measured on GB300 per step, R = 2 (marching -> tiles, equal bits): 256^2 51 -> 25 us, 384^2 67 -> 39,
+// 480^2 69 -> 53, 1000 x 200 68 -> 48; 64^2 45 -> 12 us (the launches).  At 2048^2 tiles lose:
+// 753 us against 585.
 #pragma once
 #include "plan.h"
 #include "stage.cuh"
