@@ -186,7 +186,7 @@ constexpr int kVarMean = 1, kVarFdFlux = 2, kVarAo = 4, kVarSlab = 8, kVarFlux =
 constexpr int kVarRange = 32;
 
 // Whether the smoothness indicators are divided by the square of the last form's coefficient a (beta_weight), which
-// saves an instruction per window: FP32 step of 4096^2 R = 2 2288 -> 2220 us, of 512^3 R = 3 50.7 -> 50.0 ms, HLLC R = 3
+// saves an instruction per window: FP32 step of 4096^2 R = 2 2288 -> 2220 us, of 512^3 R = 3 50.7 -> 49.8 ms, HLLC R = 3
 // 397 -> 387 us; none at R = 1 (777 x 613 25.3 us both ways).  The floor of eps + beta is divided alike (a = 1.6 at R = 2,
 // 1.1 at R = 3 for sigma = 3 dx, growing with sigma), so (eps + beta)^-p grows by a^2p.  FP32 keeps the indicators'
 // own scale where that leaves the range: in the kVarRange kernels; at R = 1 (a = 3 already); and
@@ -507,7 +507,8 @@ __device__ __forceinline__ V beta_weight(const FaceTables<T, R> &tb, const V (&d
     if constexpr (R == 3) {
         const V si = sum(1), ki = diff(1);
         s = vfma(tb.B, si, s);
-        const V m = vfma(tb.D, si, pD), n = vfma(tb.kb, t, vmul(tb.kd, ki));
+        // t is a plain copy in the two windows that end at cell s, so its product starts n (512^3 50.0 -> 49.8 ms)
+        const V m = vfma(tb.D, si, pD), n = vfma(tb.kd, ki, vmul(tb.kb, t));
         beta = vfma(m, m, beta);
         beta = vfma(n, n, beta);
     }
