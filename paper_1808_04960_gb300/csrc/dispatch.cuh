@@ -286,20 +286,22 @@ constexpr int kAnyResident = 1 << 20;   // no cap
 class Residency {
 public:
     template <typename K>
-    gpweno_status get(const gpweno_plan_s *p, K kern, int block, size_t smem, size_t smem_limit, int most, const char *what,
-                      int &ctas)
+    gpweno_status get(K kern, int block, size_t smem, size_t smem_limit, int most, const char *what, int &ctas)
     {
-        const bool cached = p->device >= 0 && p->device < kDevices;
-        ctas = cached ? of_[p->device].load(std::memory_order_acquire) : 0;
+        int device = -1;   // the current one, which the attribute is set on, also where a caller left another than the plan's
+        cudaError_t e = cudaGetDevice(&device);
+        if (e != cudaSuccess) return cuda_fail(e, what);
+        const bool cached = device >= 0 && device < kDevices;
+        ctas = cached ? of_[device].load(std::memory_order_acquire) : 0;
         if (ctas) return GPWENO_OK;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)std::max(smem, smem_limit));
         if (e != cudaSuccess) return cuda_fail(e, what);
         int n = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem);
         if (e != cudaSuccess || n < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, what);
         ctas = std::min(n, most);
-        if (cached) of_[p->device].store(ctas, std::memory_order_release);
+        if (cached) of_[device].store(ctas, std::memory_order_release);
         return GPWENO_OK;
     }
 
@@ -324,7 +326,7 @@ gpweno_status launch_stage2d_spec(gpweno_plan p, StageArgs<T> a, const TablesFor
     static Residency residency;   // per instantiation
     int occ;
     // at most MINB: R = 1's three-CTA build needs 120 registers at most and would fit four times
-    const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, MINB, "stage2d occupancy", occ);
+    const gpweno_status r = residency.get(kern, NT, smem, kSpreadSmem<T>, MINB, "stage2d occupancy", occ);
     if (r != GPWENO_OK) return r;
     Schedule s = schedule2d(a.n[0], a.n[1], NT, occ * p->num_sms);
     s.ctas_per_sm = occ;
@@ -366,7 +368,7 @@ gpweno_status launch_stagez(gpweno_plan p, const StageArgs<T> &a, const TablesFo
     auto kern = stagez_kernel<T, R, NT, VAR, SPEC>;
     static Residency residency;
     int occ;
-    const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, kAnyResident, "stagez occupancy", occ);
+    const gpweno_status r = residency.get(kern, NT, smem, kSpreadSmem<T>, kAnyResident, "stagez occupancy", occ);
     if (r != GPWENO_OK) return r;
     const long long plane = (long long)a.n[0] * a.n[1];
     const Cut3D cut = cut3d((plane + NT - 1) / NT, a.n[2], occ, p->num_sms, NT);
@@ -460,7 +462,7 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
             auto kern = plane3d_kernel<T, R, NT, VAR>;
             static Residency residency;
             int occ;
-            const gpweno_status r = residency.get(p, kern, NT, smem, kSpreadSmem<T>, kAnyResident, "plane3d occupancy", occ);
+            const gpweno_status r = residency.get(kern, NT, smem, kSpreadSmem<T>, kAnyResident, "plane3d occupancy", occ);
             if (r != GPWENO_OK) return r;
             StageArgs<T> pa = a;
             const int wmax = NT - 5;
@@ -496,7 +498,7 @@ gpweno_status launch_stage_R(gpweno_plan p, const StageArgs<T> &a0, bool use_lis
                 const size_t smem = tile2d_elems<R>(p->tile.TX, p->tile.TY) * sizeof(float4);
                 static Residency residency;   // at the largest tile; never lowered for a plan of smaller ones
                 int occ;
-                const gpweno_status r = residency.get(p, kern, NTt, kTileSmem, kTileSmem, kAnyResident, "tile2d occupancy", occ);
+                const gpweno_status r = residency.get(kern, NTt, kTileSmem, kTileSmem, kAnyResident, "tile2d occupancy", occ);
                 if (r != GPWENO_OK) return r;
                 cudaError_t e = launch_pdl(kern, p->tile.nx * p->tile.ny, NTt, smem, st, a, p->tile, tb);
                 if (e != cudaSuccess) return cuda_fail(e, "tile2d kernel launch");

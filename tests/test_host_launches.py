@@ -86,6 +86,17 @@ assert fake.fake_launches() >= 8
 """)
 
 
+def test_launch_with_another_device_current(run):
+    """Such a launch is the caller's mistake; the kernel's state on the plan's own device stays right."""
+    run("""
+p, q = plan((1024, 1024)), plan((1024, 1024))
+fake.fake_device(1)
+step(p)
+fake.fake_device(0)
+step(q)
+""")
+
+
 def test_residency_published_whole(run):
     """A second thread that launches while the first is still asking for a kernel's residency sees the final value
     (R = 1's three-CTA build would fit four times and is counted as three)."""
