@@ -79,7 +79,7 @@ struct Num<float> {
 //   1/a       = x / (1 - e) = x (1 + e + e^2 + ...),             e = 1 - a x,    |e| <= ~2^-19
 //   a^(-1/2)  = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...),  e = 1 - a y^2
 // with remainders below 2^-55: results within one unit in the last place, in 3 and 5 FP64
-// instructions (the square root in 6) in place of an IEEE division or square root plus division.  Order tests and maxima
+// instructions (the square root in 5) in place of an IEEE division or square root plus division.  Order tests and maxima
 // run on the bit patterns in the integer units.  Measured per RK3 step: 512^2 R = 2 3629 -> 3086 us,
 // 128^2 R = 3 3042 -> 2748 us; one 3D right-hand side of 70x61x45 2870 -> 2421 us.  Arguments are normal positive numbers
 // (eps + beta, densities, sums of weights); zero, infinity or NaN give NaN, which the
@@ -100,15 +100,17 @@ struct Num<double> {
         const double e = fma(-(a * y), y, 1.0);
         return fma(y * e, fma(0.375, e, 0.5), y);
     }
-    // s (1 - E)^(-1/2) = s (1 + E/2 + 3 E^2/8 + ...) with s = a y and E = (a - s^2) / a, whose numerator is exact: the same
-    // six instructions as a times rsqrt(a), which would round twice more (1.6 units in the last place; this: 0.52)
+    // Two Newton steps s + (a - s^2) y/2 from s = a y with exact residuals (relative error 2^-20 of s, 2^-39, then the last
+    // rounding): 0.51 units in the last place in five instructions, where a times rsqrt(a) takes six, rounds twice more
+    // and is up to 1.7 off.  y/2 is an integer subtraction in y's exponent.
     static __device__ __forceinline__ double sqrt(double a)
     {
         double y;
         asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-        const double s = __dmul_rn(a, y);
-        const double t = __dmul_rn(fma(-s, s, a), y);   // s E
-        return fma(t, fma(0.375, fma(-s, y, 1.0), 0.5), s);
+        const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
+        double s = __dmul_rn(a, y);
+        s = fma(fma(-s, s, a), h, s);
+        return fma(fma(-s, s, a), h, s);
     }
     // IEEE forms, zero and infinity included: once per cell, in the CFL rates
     static __device__ __forceinline__ double rcp_ieee(double x) { return 1.0 / x; }

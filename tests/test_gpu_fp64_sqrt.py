@@ -1,7 +1,7 @@
 """FP64 square root of the face kernels against extended precision, in units in the last place of the result.
 
-One third-order step from a reciprocal square root whose square is off by |E| <= 2^-18 leaves a relative remainder of at
-most (5/16) |E|^3 = (5/16) 2^-54, 0.16 units in the last place at most; with the last rounding 0.66.  Bound used: 0.7."""
+From a start of relative error d <= 2^-19 two Newton steps with a slope 1/(2 s) that is as far off leave d^2 (3/2) and then
+d^3 (3/2) <= 2^-56, 0.13 units in the last place at most; with the last rounding 0.63.  Bound used: 0.7."""
 import ctypes
 import subprocess
 
